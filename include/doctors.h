@@ -93,8 +93,8 @@ typedef struct doctors_options {
     int angles_per_block;    /* directions per sweep block (0 = default: whole octants on the dataflow
                                 sweep, else the largest of 12, 10, 9, 7, ... dividing it); must divide
                                 N(N+2)/8; 21 and 36 (whole S12, S16 octants) on the dataflow sweep only */
-    int sweep_kernel;        /* 0 = default (the fastest measured: dataflow with a face warp (7) where
-                                it applies, else plain dataflow (4), else chained (3)),
+    int sweep_kernel;        /* 0 = default (the fastest measured: dataflow (4, 7) where it applies,
+                                else chained (3)),
                                 1 = CUDA-core transforms, one task (tile, octant, direction block,
                                 group) per CTA, 3 = CUDA-core transforms, each CTA running a chain of
                                 tasks of a stage back to back in one hyperplane pipeline,
@@ -109,9 +109,9 @@ typedef struct doctors_options {
                                 writes one angular record per cell, a pass turns the angular fluence
                                 back into moments (whole octants of S2..S8 only; two more arrays
                                 of G x N(N+2) x V floats, padded),
-                                7 = dataflow with a face warp: one more warp per CTA fetches and
-                                waits for the incoming face fluxes, the column threads only sweep
-                                (same conditions as 4, P1 or P3, tile_x + tile_y <= 64),
+                                7 = the same kernel as 4 (one warp per CTA fetches and waits for
+                                the incoming face fluxes, the column threads only sweep), taken
+                                only for P1 or P3 and tile_x + tile_y <= 64,
                                 8 = as 5 with the two transform passes on the tensor cores
                                 (tcgen05, 3xTF32 with FP32 accumulation; P3 only).
                                 2 and 6 are not offered (DOCTORS_ERR_INVALID_ARG): a sweep with
@@ -349,7 +349,7 @@ typedef struct doctors_tuning {
     int tile_x, tile_y;      /* tile of columns */
     int angles_per_block;    /* directions per CTA */
     int sweep_kernel;        /* 1 CUDA-core, 3 chained, 4 dataflow, 5 dataflow with split transforms,
-                                7 dataflow with a face warp, 8 split transforms on the tensor cores
+                                7 dataflow (as 4), 8 split transforms on the tensor cores
                                 (as doctors_options) */
     double ms_per_sweep;     /* measured time of one full sweep of this problem */
     int candidates;          /* schedules timed (0 if taken from the cache) */

@@ -25,7 +25,7 @@ def main():
     ap.add_argument("--tile", type=int, nargs=2, default=(0, 0))
     ap.add_argument("--ab", type=int, default=0)
     ap.add_argument("--kernel", type=int, default=0, help="sweep kernel: 0 default, 1 CUDA-core, 3 chained CUDA-core, 4 dataflow, 5 dataflow with split "
-                    "transforms, 7 dataflow with a face warp, 8 split transforms on the tensor cores")
+                    "transforms, 7 dataflow (as 4), 8 split transforms on the tensor cores")
     ap.add_argument("--sn", type=int, default=None, help="quadrature order (tiny_cube, water_cylinder, abdomen)")
     ap.add_argument("--legendre", type=int, default=None, help="Legendre order (tiny_cube, water_cylinder, abdomen)")
     ap.add_argument("--device-loop", action="store_true",

@@ -253,11 +253,12 @@ SweepArgs sweep_args(const doctors_problem* p, int reverse, const float* src, fl
     a.g0 = 0;
     a.gcount = p->G;
     a.chain_slots = p->chain_slots;
+    a.depth = p->flow_depth;
+    a.fpitch = p->face_pitch;
     a.dir_table = &p->dir_table;
     a.flow = (p->use_flow || p->use_split) ? p->d_flow : nullptr;
     a.qang = p->d_qang;
     a.pang = p->d_pang;
-    a.hw = p->flow_hw ? 1 : 0;
     a.tc_b1 = (p->use_split && p->split_tc) ? p->d_tcb : nullptr;
     a.tc_b2 = (p->use_split && p->split_tc) ? p->d_tcb + p->tcb1_floats : nullptr;
     a.dd = p->differencing == DOCTORS_DIFF_DIAMOND ? 1 : 0;
@@ -270,9 +271,8 @@ SweepArgs sweep_args(const doctors_problem* p, int reverse, const float* src, fl
 cudaError_t launch_sweep(const doctors_problem* p, SweepArgs sw, int mode, cudaStream_t s, int* count) {
     if (p->use_split && mode == 0) return launch_split_sweep(sw, p->M, s, count);
     if (p->use_flow || p->use_split) {
-        // modes 1 and 2 (stored / paired angular fluence) of the split and face-warp
-        // paths use the plain dataflow kernel
-        if (p->use_split || (mode != 0 && p->flow_hw)) sw.chain_slots = p->flow_slots;
+        // modes 1 and 2 (stored / paired angular fluence) of the split path use the fused kernel
+        if (p->use_split) sw.chain_slots = p->flow_slots;
         if (p->nab == 1) {
             *count = 1;
             return launch_sweep_flow(sw, p->M, mode, s);
@@ -675,18 +675,32 @@ int configure_sweep(doctors_problem* p, int tx, int ty, int ab, int kernel) {
         return DOCTORS_ERR_INVALID_ARG;
     }
     const int ntx = (p->nx + tx - 1) / tx, nty = (p->ny + ty - 1) / ty;
-    int chain_slots = 0, flow_slots = 0;
+    int chain_slots = 0, flow_slots = 0, flow_depth = 2;
     size_t smem = 0;
     if (use_flow || use_split) {
         int sms = 0;
         CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device));
-        smem = sweep_flow_smem_bytes(ab, tx, ty, p->G, kMaxMat, dd);
+        // pipeline depth: four steps of source and face records in flight cover the
+        // L2 latency (96x80x24, 10 groups, S2 P1: 0.380 ms per sweep at depth 4 and
+        // 0.511 at 2), unless their shared memory costs resident CTAs (cylinder, S8
+        // P3, 16x8 tiles: 0.85 ms at depth 4 with three CTAs per SM, 0.78 at depth 2
+        // with four) or does not fit at all
+        const int threads = flow_threads(tx, ty);
+        int per_sm = 0, per_sm_main = 0;
+        for (int depth = 2; depth <= 4; depth += 2) {
+            const size_t sf = sweep_flow_smem_bytes(ab, p->M, tx, ty, p->G, depth, dd);
+            const size_t ss = use_split ? sweep_flow_smem_bytes(ab, flow_abp_host(ab), tx, ty, p->G, depth) : 0;
+            if (depth == 2) smem = std::max(sf, ss);
+            if (std::max(sf, ss) > 227 * 1024) break;
+            const int b = sweep_flow_blocks_per_sm(ab, p->M, threads, sf, false, dd);
+            const int bm = use_split ? sweep_flow_blocks_per_sm(ab, p->M, threads, ss, true) : b;
+            if (depth == 2 || (b >= per_sm && bm >= per_sm_main)) {
+                per_sm = b;
+                per_sm_main = bm;
+                flow_depth = depth;
+            }
+        }
         if (smem <= 227 * 1024) {
-            const int per_sm = sweep_flow_blocks_per_sm(ab, p->M, tx * ty, smem, false, dd);
-            const int hw_threads = ((tx * ty + 31) / 32 + 1) * 32;
-            const int per_sm_main = use_split ? sweep_flow_blocks_per_sm(ab, p->M, tx * ty, smem, true)
-                                  : hw ? sweep_flow_blocks_per_sm(ab, p->M, hw_threads, smem, false, false, true)
-                                       : per_sm;
             if (per_sm < 1 || per_sm_main < 1) {
                 set_error("dataflow sweep cannot be resident with this tile");
                 return DOCTORS_ERR_INVALID_ARG;
@@ -721,26 +735,28 @@ int configure_sweep(doctors_problem* p, int tx, int ty, int ab, int kernel) {
         return DOCTORS_ERR_INVALID_ARG;
     }
     // face buffers: [8][A/8][G][tiles-1][ny or nx][nz] per direction for the
-    // staged kernels; [8][G][tiles-1][ny or nx][nz][A/8 padded to 4] records
-    // for the dataflow kernel
-    const size_t per_dir = std::max((size_t)p->A, (size_t)8 * flow_abp_host(p->A8));
-    const size_t xf = per_dir * p->G * (ntx > 1 ? ntx - 1 : 0) * p->ny * p->nz;
-    const size_t yf = per_dir * p->G * (nty > 1 ? nty - 1 : 0) * p->nx * p->nz;
-    if (p->d_xface == nullptr || xf * sizeof(float) > p->xface_bytes) {
-        float* nb = nullptr;
-        int rc = dalloc_t(&nb, xf, "x face buffer");
-        if (rc) return rc;
-        if (p->d_xface) cudaFree(p->d_xface);
-        p->d_xface = nb;
-        p->xface_bytes = xf * sizeof(float);
-    }
-    if (p->d_yface == nullptr || yf * sizeof(float) > p->yface_bytes) {
-        float* nb = nullptr;
-        int rc = dalloc_t(&nb, yf, "y face buffer");
-        if (rc) return rc;
-        if (p->d_yface) cudaFree(p->d_yface);
-        p->d_yface = nb;
-        p->yface_bytes = yf * sizeof(float);
+    // staged kernels; [8][G][tiles-1][ny or nx][nz] records of `pitch` floats for
+    // the dataflow kernels (unpadded records where padded ones do not fit)
+    int pitch = use_flow || use_split ? flow_face_pitch(ab) : flow_abp_host(p->A8);
+    for (;;) {
+        const size_t per_dir = std::max((size_t)p->A, (size_t)8 * std::max(pitch, flow_abp_host(p->A8)));
+        const size_t xf = per_dir * p->G * (ntx > 1 ? ntx - 1 : 0) * p->ny * p->nz;
+        const size_t yf = per_dir * p->G * (nty > 1 ? nty - 1 : 0) * p->nx * p->nz;
+        auto grow = [&](float** buf, size_t* bytes, size_t n, const char* what) -> int {
+            if (*buf != nullptr && n * sizeof(float) <= *bytes) return DOCTORS_OK;
+            float* nb = nullptr;
+            const int rc = dalloc_t(&nb, n, what);
+            if (rc) return rc;
+            if (*buf) cudaFree(*buf);
+            *buf = nb;
+            *bytes = n * sizeof(float);
+            return DOCTORS_OK;
+        };
+        int rc = grow(&p->d_xface, &p->xface_bytes, xf, "x face buffer");
+        if (!rc) rc = grow(&p->d_yface, &p->yface_bytes, yf, "y face buffer");
+        if (!rc) break;
+        if (rc != DOCTORS_ERR_OOM || pitch == flow_abp_host(ab)) return rc;
+        pitch = flow_abp_host(ab);
     }
     if (use_split) {
         // angular source and fluence records of every direction, group and voxel
@@ -786,6 +802,8 @@ int configure_sweep(doctors_problem* p, int tx, int ty, int ab, int kernel) {
     p->flow_hw = use_flow && hw;
     p->chain_slots = chain_slots;
     p->flow_slots = flow_slots;
+    p->flow_depth = flow_depth;
+    p->face_pitch = pitch;
     return DOCTORS_OK;
 }
 
@@ -1290,6 +1308,8 @@ int doctors_autotune(doctors_problem* p, doctors_tuning* out) {
                 if ((kernel == 1 || kernel == 3) && !sweep_supported(ab, p->M)) continue;
                 if ((kernel == 5 || kernel == 8) && !(p->A8 == ab && chain_const_table_ab(ab))) continue;
                 if ((kernel == 4 || kernel == 7) && !flow_block_ab(p->A8, ab)) continue;
+                // 4 and 7 are the same kernel: one of them is timed
+                if (kernel == 4 && p->M % 4 == 0 && p->differencing != DOCTORS_DIFF_DIAMOND && t[0] + t[1] <= 64) continue;
                 if (configure_sweep(p, t[0], t[1], ab, kernel) != DOCTORS_OK) continue;
                 SweepArgs sw = sweep_args(p, 0, p->d_Q, p->d_mom);
                 float total = 0.0f;

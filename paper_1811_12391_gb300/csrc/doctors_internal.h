@@ -191,6 +191,9 @@ struct SweepArgs {
     float* psi;                        // written (mode 1) or read (mode 2): [G][V][A], dataflow kernel [G][V][8][ABP]
     float* prod;                       // [G][V]: mode 2 accumulator
     const int* skip;                   // if non-null and *skip != 0 the kernel does nothing
+    int depth;                         // dataflow kernels: steps of source and face records held in shared memory
+                                       // (fetched depth - 1 and depth steps ahead; 2 or 4)
+    int fpitch;                        // dataflow kernels: floats from one face record to the next
     int chain_slots;                   // > 0: chained kernel, at most this many CTAs per stage launch
     const int* win;                    // dataflow kernels: non-null: sweep the groups [win[0], win[1]) read from
                                        // device memory (g0, gcount then give only the buffer layout)
@@ -199,8 +202,6 @@ struct SweepArgs {
     const struct ChainDirTable* dir_table;   // host copy of the first-octant direction table (chained kernel)
     const float* qang;                 // split transforms: angular source [G][8][V][ABP] (direction octant)
     float* pang;                       // split transforms: angular fluence [G][8][V][ABP]
-    int hw;                            // dataflow kernel: 1 = a face warp per CTA takes the incoming
-                                       // face records (mode 0)
     const float* tc_b1;                // split transforms on the tensor cores (P3): moments -> directions
     const float* tc_b2;                // and directions -> moments operand tables, or null
     int dd;                            // dataflow kernel: 1 = diamond differencing (dir_table holds 2c), 0 = step
@@ -270,21 +271,36 @@ inline size_t sweep_chain_smem_bytes(int ab, int tx, int ty, int cmax, int gcoun
     return 16 * (size_t)cmax * ab * 5 + 8 * (size_t)gcount +
            4 * ((size_t)2 * chain_rs(ab) * chain_px(tx) * (ty + 1) + (size_t)cmax * ab + (size_t)gcount * nmat);
 }
-// shared memory of one dataflow-sweep CTA: the fetched face records of the
-// tile's first row and column, per-group leakage, the two halo-padded
-// hyperplanes, sigma_t of the swept groups and the task slot
-inline int flow_abp_host(int ab) { return (ab + 3) & ~3; }
-inline size_t sweep_flow_smem_bytes(int ab, int tx, int ty, int gcount, int nmat, bool dd = false) {
-    // prefetched source moments (2 slots of 16 floats per thread), two landing
-    // slots (pipeline depth 2) of one record per edge column, the leakage per
-    // group, two planes of column records (diamond differencing: x-going and
-    // y-going face fluxes in separate planes), the cross sections and the task slot
-    return 2 * (size_t)16 * 4 * (size_t)tx * ty + 2 * (size_t)4 * (tx + ty) * flow_abp_host(ab) +
-           8 * (size_t)gcount +
-           4 * ((size_t)(dd ? 4 : 2) * chain_rs(ab) * chain_px(tx) * (ty + 1) + (size_t)gcount * nmat) + 16;
+// Dataflow sweep.  A column's AB fluxes are one plane record of flow_rs(AB)
+// floats, read and written as vectors of flow_pw(AB) floats; a record is an
+// odd number of vectors, so the threads of a tile diagonal (an odd number of
+// records apart) fall in distinct shared-memory banks at that width.
+__host__ __device__ constexpr int flow_abp_host(int ab) { return (ab + 3) & ~3; }
+// floats from one face record to the next: whole 32-byte sectors for the
+// 16-byte records of S2 and S4 (a record that shares its sector with the one
+// its producer writes next is slow to read: S2 P0, 96x80x24, 10 groups takes
+// 0.331 ms per sweep at 16 bytes and 0.196 at 32; at 8 and more fluxes per
+// record padding only adds traffic: S8 P3 0.748 at 48 bytes, 0.760 at 64)
+__host__ __device__ constexpr int flow_face_pitch(int ab) { return ab <= 4 ? 8 : (ab + 3) & ~3; }
+__host__ __device__ constexpr int flow_pw(int ab) { return ab == 1 ? 1 : (flow_abp_host(ab) / 4) % 2 == 1 ? 4 : 2; }
+__host__ __device__ constexpr int flow_rs(int ab) {
+    return flow_pw(ab) == 4 ? flow_abp_host(ab) : flow_pw(ab) == 2 ? (((ab + 1) / 2) | 1) * 2 : 1;
 }
-int sweep_flow_blocks_per_sm(int ab, int M, int threads, size_t smem, bool split = false, bool dd = false,
-                             bool hw = false);
+__host__ __device__ constexpr int flow_up4(int n) { return (n + 3) & ~3; }
+// column threads in whole warps, then the face warp
+inline int flow_threads(int tx, int ty) { return ((tx * ty + 31) / 32 + 1) * 32; }
+// shared memory of one dataflow-sweep CTA: the source records (rf floats) and
+// cross sections of `depth` steps, the fetched face records of the tile's
+// first row and column of as many steps, two
+// halo-padded hyperplanes (diamond differencing: x-going and y-going face
+// fluxes in separate planes), per-group leakage and the task slot
+inline size_t sweep_flow_smem_bytes(int ab, int rf, int tx, int ty, int gcount, int depth, bool dd = false) {
+    const int T = tx * ty;
+    return 4 * ((size_t)flow_up4(depth * T * rf) + flow_up4(depth * T) + (size_t)depth * (tx + ty) * flow_abp_host(ab) +
+                flow_up4((dd ? 4 : 2) * chain_px(tx) * (ty + 1) * flow_rs(ab))) +
+           8 * (size_t)gcount + 16;
+}
+int sweep_flow_blocks_per_sm(int ab, int M, int threads, size_t smem, bool split = false, bool dd = false);
 cudaError_t launch_sweep_flow(const SweepArgs& a, int M, int mode, cudaStream_t s);
 // split transforms (whole octants of S2..S8): moments -> angular source for
 // all 8 octants, the dataflow sweep on angular records (a.qang -> a.pang),
@@ -340,9 +356,11 @@ struct doctors_problem {
     bool use_flow = false;          // dataflow sweep (one launch per sweep, task queue)
     bool use_split = false;         // dataflow sweep with the transforms in separate passes
     bool split_tc = false;          // ... those passes on the tensor cores (P3)
-    bool flow_hw = false;           // dataflow sweep: a face warp per CTA
+    bool flow_hw = false;           // dataflow sweep chosen as sweep_kernel 7 (the same kernel as 4)
     int differencing = 0;           // DOCTORS_DIFF_STEP or DOCTORS_DIFF_DIAMOND
-    int flow_slots = 0;             // CTA slots of the plain dataflow kernel (modes 1, 2 under split)
+    int flow_depth = 2;             // dataflow sweep: pipeline depth (SweepArgs::depth)
+    int face_pitch = 4;             // dataflow sweep: floats from one face record to the next
+    int flow_slots = 0;             // CTA slots of the fused dataflow kernel (modes 1, 2 under split)
     float* d_qang = nullptr;        // [G][8][V][ABP] angular source (split)
     float* d_pang = nullptr;        // [G][8][V][ABP] angular fluence (split)
     float* d_tcb = nullptr;         // split transforms on the tensor cores: operand tables b1, b2

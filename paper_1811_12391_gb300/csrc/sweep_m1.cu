@@ -28,8 +28,8 @@ cudaError_t launch_sweep_flow_m1_entry(const SweepArgs& a, int mode, cudaStream_
         default: return cudaErrorInvalidValue;
     }
 }
-int sweep_flow_blocks_m1(int ab, int threads, size_t smem, bool split, bool dd, bool hw) {
-    return sweep_flow_blocks_per_sm<1>(ab, threads, smem, split, dd, hw);
+int sweep_flow_blocks_m1(int ab, int threads, size_t smem, bool split, bool dd) {
+    return sweep_flow_blocks_per_sm<1>(ab, threads, smem, split, dd);
 }
 cudaError_t launch_split_sweep_m1_entry(const SweepArgs& a, cudaStream_t s, int* count) {
     return launch_split_sweep_m<1>(a, s, count);
