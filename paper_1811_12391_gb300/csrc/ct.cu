@@ -6,12 +6,20 @@
 // between ascending thresholds, and a density piecewise linear in the CT
 // number through ascending knots, constant beyond the end knots.
 //
-// One thread per voxel (grid-stride over a resident grid); the calibration
-// is a kernel parameter, read through the constant bank.  The density is
-// formed with explicitly rounded FP32 operations in a fixed order, so a
-// plain FP32 evaluation of the same steps gives the same bits.  HBM-bound:
-// 4 bytes read and 5 written per voxel.
+// Bins and segments are found by counting thresholds and knots (kernel
+// parameters read at uniform indices, so they come from the constant bank);
+// what a voxel then looks up by its own bin and segment comes from shared
+// memory, where the lanes of a warp may differ.  The density is formed with
+// explicitly rounded FP32 operations in a fixed order, so a plain FP32
+// evaluation of the same steps gives the same bits.  A thread takes four
+// neighbouring voxels (16-byte loads and stores) where the arrays are aligned.
+// Floor: 4 bytes read and 5 written per voxel, 56 us at the measured copy rate
+// for a 512 x 512 x 160 volume, which takes 105 us (bound by the compares and
+// the division; 285 us with one voxel per thread and per-lane constant indices,
+// where a constant load is replayed once per distinct index in the warp).
+#include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <string>
 
 #include "doctors_internal.h"
@@ -29,29 +37,66 @@ struct CtCalib {
     float hk[kCtMaxKnots], rk[kCtMaxKnots];  // density knots (CT number, density)
 };
 
+template <int VEC>
 __global__ void __launch_bounds__(256) k_ct_to_materials(const float* __restrict__ hu, size_t n, const CtCalib c,
                                                          uint8_t* __restrict__ mat, float* __restrict__ rho) {
-    for (size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (size_t)gridDim.x * blockDim.x) {
-        const float h = hu[v];
-        // bin: the number of thresholds at or below h (NaN: bin 0)
-        int b = 0;
-        for (int i = 0; i < c.nt; ++i) b += c.t[i] <= h ? 1 : 0;
-        // density: the number of knots at or below h picks the segment
-        int k = 0;
-        for (int i = 0; i < c.nk; ++i) k += c.hk[i] <= h ? 1 : 0;
-        float r;
-        if (k == 0) {
-            r = c.rk[0];                       // below the first knot, or NaN
-        } else if (k == c.nk) {
-            r = c.rk[c.nk - 1];                // at or beyond the last knot
-        } else {
-            const int s = k - 1;               // hk[s] <= h < hk[s + 1]
-            const float t = __fdiv_rn(__fsub_rn(h, c.hk[s]), __fsub_rn(c.hk[s + 1], c.hk[s]));
-            r = __fadd_rn(c.rk[s], __fmul_rn(t, __fsub_rn(c.rk[s + 1], c.rk[s])));
-        }
-        mat[v] = c.m[b];
-        rho[v] = r;
+    // segment k (knots at or below the voxel's number): knot, spacing, density, rise
+    __shared__ float4 seg[kCtMaxKnots + 1];
+    __shared__ uint8_t bin[kCtMaxThresholds + 1];
+    for (int k = threadIdx.x; k <= c.nk; k += blockDim.x) {
+        if (k == 0) seg[k] = make_float4(0.0f, 1.0f, c.rk[0], 0.0f);                    // below the first knot, or NaN
+        else if (k == c.nk) seg[k] = make_float4(0.0f, 1.0f, c.rk[c.nk - 1], 0.0f);     // at or beyond the last knot
+        else seg[k] = make_float4(c.hk[k - 1], __fsub_rn(c.hk[k], c.hk[k - 1]), c.rk[k - 1], __fsub_rn(c.rk[k], c.rk[k - 1]));
     }
+    for (int i = threadIdx.x; i <= c.nt; i += blockDim.x) bin[i] = c.m[i];
+    __syncthreads();
+    const size_t nv = n / VEC;
+    for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < nv; q += (size_t)gridDim.x * blockDim.x) {
+        float h[VEC], r[VEC];
+        if constexpr (VEC == 4) {
+            const float4 t = __ldcs(reinterpret_cast<const float4*>(hu) + q);
+            h[0] = t.x; h[1] = t.y; h[2] = t.z; h[3] = t.w;
+        } else {
+            h[0] = hu[q];
+        }
+        // bin: the number of thresholds at or below h (NaN: bin 0); segment: the number of knots
+        int b[VEC], k[VEC];
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) b[e] = k[e] = 0;
+        for (int i = 0; i < c.nt; ++i)
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) b[e] += c.t[i] <= h[e] ? 1 : 0;
+        for (int i = 0; i < c.nk; ++i)
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) k[e] += c.hk[i] <= h[e] ? 1 : 0;
+        unsigned m = 0;
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) {
+            const float4 g = seg[k[e]];
+            const float t = __fdiv_rn(__fsub_rn(h[e], g.x), g.y);
+            r[e] = k[e] == 0 || k[e] == c.nk ? g.z : __fadd_rn(g.z, __fmul_rn(t, g.w));
+            m |= (unsigned)bin[b[e]] << (8 * e);
+        }
+        if constexpr (VEC == 4) {
+            __stcs(reinterpret_cast<unsigned*>(mat) + q, m);
+            __stcs(reinterpret_cast<float4*>(rho) + q, make_float4(r[0], r[1], r[2], r[3]));
+        } else {
+            mat[q] = (uint8_t)m;
+            rho[q] = r[0];
+        }
+    }
+}
+
+// the vector form for the aligned whole fours, the scalar one for the rest
+cudaError_t launch_ct(const float* hu, size_t n, const CtCalib& c, uint8_t* mat, float* rho, int nsm, cudaStream_t s) {
+    const size_t cap = (size_t)nsm * 8;
+    auto blocks = [&](size_t k) { return (unsigned)std::min<size_t>((k + 255) / 256, cap); };
+    const bool aligned = ((reinterpret_cast<uintptr_t>(hu) | reinterpret_cast<uintptr_t>(rho)) & 15) == 0 &&
+                         (reinterpret_cast<uintptr_t>(mat) & 3) == 0;
+    const size_t n4 = aligned ? n & ~(size_t)3 : 0;
+    if (n4 > 0) k_ct_to_materials<4><<<blocks(n4 / 4), 256, 0, s>>>(hu, n4, c, mat, rho);
+    if (n > n4) k_ct_to_materials<1><<<blocks(n - n4), 256, 0, s>>>(hu + n4, n - n4, c, mat + n4, rho + n4);
+    return cudaGetLastError();
 }
 
 int fail(int code, const std::string& msg) {
@@ -99,11 +144,8 @@ extern "C" int doctors_ct_to_materials(const float* hu, size_t n, int n_threshol
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return fail(DOCTORS_ERR_CUDA, std::string("doctors_ct_to_materials: ") + cudaGetErrorString(e));
-    const size_t want = (n + 255) / 256, cap = (size_t)nsm * 8;
-    const unsigned grid = (unsigned)(want < cap ? want : cap);
     if (mem == DOCTORS_MEM_DEVICE) {
-        k_ct_to_materials<<<grid, 256, 0, s>>>(hu, n, c, mat_out, rho_out);
-        e = cudaGetLastError();
+        e = launch_ct(hu, n, c, mat_out, rho_out, nsm, s);
         if (e != cudaSuccess)
             return fail(DOCTORS_ERR_CUDA, std::string("doctors_ct_to_materials: ") + cudaGetErrorString(e));
         return DOCTORS_OK;
@@ -123,10 +165,7 @@ extern "C" int doctors_ct_to_materials(const float* hu, size_t n, int n_threshol
         return fail(DOCTORS_ERR_OOM, "doctors_ct_to_materials: device buffers");
     }
     e = cudaMemcpyAsync(d_hu, hu, n * sizeof(float), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) {
-        k_ct_to_materials<<<grid, 256, 0, s>>>(d_hu, n, c, d_mat, d_rho);
-        e = cudaGetLastError();
-    }
+    if (e == cudaSuccess) e = launch_ct(d_hu, n, c, d_mat, d_rho, nsm, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(mat_out, d_mat, n, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(rho_out, d_rho, n * sizeof(float), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
