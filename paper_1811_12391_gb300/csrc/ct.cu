@@ -50,14 +50,16 @@ __global__ void __launch_bounds__(256) k_ct_to_materials(const float* __restrict
     }
     for (int i = threadIdx.x; i <= c.nt; i += blockDim.x) bin[i] = c.m[i];
     __syncthreads();
-    const size_t nv = n / VEC;
+    const size_t nv = (n + VEC - 1) / VEC;
     for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < nv; q += (size_t)gridDim.x * blockDim.x) {
         float h[VEC], r[VEC];
-        if constexpr (VEC == 4) {
+        const size_t left = n - q * VEC;          // the last vector may be short
+        if (VEC == 4 && left >= 4) {
             const float4 t = __ldcs(reinterpret_cast<const float4*>(hu) + q);
-            h[0] = t.x; h[1] = t.y; h[2] = t.z; h[3] = t.w;
+            h[0] = t.x; h[1 % VEC] = t.y; h[2 % VEC] = t.z; h[3 % VEC] = t.w;
         } else {
-            h[0] = hu[q];
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) h[e] = e < left ? hu[q * VEC + e] : 0.0f;
         }
         // bin: the number of thresholds at or below h (NaN: bin 0); segment: the number of knots
         int b[VEC], k[VEC];
@@ -77,25 +79,28 @@ __global__ void __launch_bounds__(256) k_ct_to_materials(const float* __restrict
             r[e] = k[e] == 0 || k[e] == c.nk ? g.z : __fadd_rn(g.z, __fmul_rn(t, g.w));
             m |= (unsigned)bin[b[e]] << (8 * e);
         }
-        if constexpr (VEC == 4) {
+        if (VEC == 4 && left >= 4) {
             __stcs(reinterpret_cast<unsigned*>(mat) + q, m);
-            __stcs(reinterpret_cast<float4*>(rho) + q, make_float4(r[0], r[1], r[2], r[3]));
+            __stcs(reinterpret_cast<float4*>(rho) + q, make_float4(r[0], r[1 % VEC], r[2 % VEC], r[3 % VEC]));
         } else {
-            mat[q] = (uint8_t)m;
-            rho[q] = r[0];
+#pragma unroll
+            for (int e = 0; e < VEC; ++e)
+                if (e < left) {
+                    mat[q * VEC + e] = (uint8_t)(m >> (8 * e));
+                    rho[q * VEC + e] = r[e];
+                }
         }
     }
 }
 
-// the vector form for the aligned whole fours, the scalar one for the rest
+// four voxels per thread where the arrays are aligned
 cudaError_t launch_ct(const float* hu, size_t n, const CtCalib& c, uint8_t* mat, float* rho, int nsm, cudaStream_t s) {
     const size_t cap = (size_t)nsm * 8;
     auto blocks = [&](size_t k) { return (unsigned)std::min<size_t>((k + 255) / 256, cap); };
     const bool aligned = ((reinterpret_cast<uintptr_t>(hu) | reinterpret_cast<uintptr_t>(rho)) & 15) == 0 &&
                          (reinterpret_cast<uintptr_t>(mat) & 3) == 0;
-    const size_t n4 = aligned ? n & ~(size_t)3 : 0;
-    if (n4 > 0) k_ct_to_materials<4><<<blocks(n4 / 4), 256, 0, s>>>(hu, n4, c, mat, rho);
-    if (n > n4) k_ct_to_materials<1><<<blocks(n - n4), 256, 0, s>>>(hu + n4, n - n4, c, mat + n4, rho + n4);
+    if (aligned) k_ct_to_materials<4><<<blocks((n + 3) / 4), 256, 0, s>>>(hu, n, c, mat, rho);
+    else k_ct_to_materials<1><<<blocks(n), 256, 0, s>>>(hu, n, c, mat, rho);
     return cudaGetLastError();
 }
 
