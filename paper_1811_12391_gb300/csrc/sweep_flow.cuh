@@ -125,6 +125,32 @@ __device__ __forceinline__ void store_record(float* p, const float (&v)[AB]) {
                               4 * c4 + 3 < AB ? v[4 * c4 + 3 < AB ? 4 * c4 + 3 : 0] : 0.0f);
 }
 
+// sum of N products, two at a time: the two lanes of packed operations, and
+// their sum
+template <int N>
+__device__ __forceinline__ float2 dot2(const float* c, const float* x) {
+    float2 t = N == 1 ? make_float2(c[0] * x[0], 0.0f) : make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int k = 0; k + 1 < N; k += 2) t = __ffma2_rn(make_float2(c[k], c[k + 1]), make_float2(x[k], x[k + 1]), t);
+    if constexpr (N % 2 == 1 && N > 1) t.x = fmaf(c[N - 1], x[N - 1], t.x);
+    return t;
+}
+template <int N>
+__device__ __forceinline__ float dot(const float* c, const float* x) {
+    if constexpr (N == 1) return c[0] * x[0];
+    const float2 t = dot2<N>(c, x);
+    return t.x + t.y;
+}
+
+// sign of R_lm under the reflections (fx, fy, fz) = +-1
+__device__ __forceinline__ float sign_lm(int lm, float fx, float fy, float fz) {
+    float r = 1.0f;
+    if ((kOddX >> lm) & 1u) r *= fx;
+    if ((kOddY >> lm) & 1u) r *= fy;
+    if ((kOddZ >> lm) & 1u) r *= fz;
+    return r;
+}
+
 // column (li, lj) of column thread t: the tile's columns in diagonal order
 __device__ __forceinline__ void flow_column(int t, int tx, int ty, int& li, int& lj) {
     int base = 0;
@@ -164,7 +190,7 @@ __device__ __forceinline__ int flow_stage_tiles(int s, int ntx, int nty) {
 // columns) or 288.  The register file is shared out by warps per scheduler, so
 // a bound of 288 threads leaves at most 168 registers (96 for two CTAs).
 template <int AB, int M, int MODE, bool SPLIT, bool DD, int NT>
-__global__ void __launch_bounds__(NT, NT == 96 ? (AB > 21 ? 2 : AB > 12 ? 3 : kFlowMinCtas) : AB > 12 ? 1 : 2)
+__global__ void __launch_bounds__(NT, NT == 96 ? (AB > 12 ? 4 : kFlowMinCtas) : AB > 12 ? 1 : 2)
     k_sweep_flow(const SweepArgs a, const ChainDirTable dt) {
     static_assert(!SPLIT || MODE == 0, "split transforms sweep in mode 0 only");
     static_assert(!DD || !SPLIT, "diamond differencing in the fused kernel only");
@@ -173,6 +199,8 @@ __global__ void __launch_bounds__(NT, NT == 96 ? (AB > 21 ? 2 : AB > 12 ? 3 : kF
     constexpr int RS = flow_rs(AB), PW = flow_pw(AB);   // plane record: floats, vector width
     constexpr int RF = SPLIT ? ABP : M;                 // floats of a cell's source record
     constexpr bool COOP = RF == 16;                     // record moved by four lanes
+    constexpr bool SWAP = !SPLIT && flow_swap(AB, M);      // transforms in even and odd parts
+    constexpr int NPR = flow_pairs(AB), NE_ = flow_even(AB, M), NO_ = flow_odd(AB, M);
     extern __shared__ float4 sm4[];
     if (a.skip && *a.skip) return;          // retired instance of a batched loop
     const int PX = chain_px(a.tx);
@@ -195,21 +223,30 @@ __global__ void __launch_bounds__(NT, NT == 96 ? (AB > 21 ? 2 : AB > 12 ? 3 : kF
         g0 = a.win[0];
         gcount = a.win[1] - a.win[0];
     }
-    const int tid = threadIdx.x, lane = tid & 31;
-    for (int e = tid; e < gcount; e += blockDim.x) leak_s[e] = 0.0;
-    for (int e = tid; e < (DD ? 4 : 2) * P * RS; e += blockDim.x) buf[e] = 0.0f;
+    for (int e = threadIdx.x; e < gcount; e += blockDim.x) leak_s[e] = 0.0;
+    for (int e = threadIdx.x; e < (DD ? 4 : 2) * P * RS; e += blockDim.x) buf[e] = 0.0f;
 
-    const bool fw = tid >= ((T + 31) & ~31);                  // the face warp: the last one
+    // The face warp is the CTA's first or last warp, by the warp slot the CTA
+    // starts at: the slots go round the SM's four schedulers, and this way the
+    // column warps of successive three-warp CTAs take schedulers 1, 2 and 3, 0
+    // in turn, so that an even number of CTAs loads them evenly
+    unsigned wslot;
+    asm volatile("mov.u32 %0, %%warpid;" : "=r"(wslot));
+    if (threadIdx.x == 0) task_s[1] = (int)(wslot & 1);
+    __syncthreads();
+    const int nwarps = (int)(blockDim.x >> 5), wid = (int)(threadIdx.x >> 5);
+    const int fwarp = task_s[1] ? nwarps - 1 : 0;
+    const bool fw = wid == fwarp;
+    const int tid = (int)threadIdx.x - (wid > fwarp ? 32 : 0), lane = threadIdx.x & 31;   // column threads: 0 .. T - 1
     const unsigned nxy = (unsigned)a.nx * a.ny;
     const size_t V = (size_t)nxy * a.nz;
-    const int nst = a.ntx + a.nty - 1;
     const int ntxf = a.ntx > 1 ? a.ntx - 1 : 0, ntyf = a.nty > 1 ? a.nty - 1 : 0;
     const size_t xslab = (size_t)a.ny * a.nz * FP, yslab = (size_t)a.nx * a.nz * FP;
     const int ntasks = a.ntx * a.nty * 8 * gcount;
     const int hend = a.nz + a.tx + a.ty - 2;                  // steps of a task
 
     // threads own the tile's columns in diagonal order (li + lj ascending)
-    const bool colthread = tid < T;
+    const bool colthread = !fw && tid < T;
     int li = 0, lj = 0;
     if (colthread) flow_column(tid, a.tx, a.ty, li, lj);
     const int d = li + lj;
@@ -229,7 +266,7 @@ __global__ void __launch_bounds__(NT, NT == 96 ? (AB > 21 ? 2 : AB > 12 ? 3 : kF
     float lk = 0.0f;
     int stage = 0, sbase = 0;                 // stage of the CTA's current task and its first task
     const int hook = a.flow[3] - 1;           // test hook: this task owes no faces
-    if (tid == 0) *task_s = atomicAdd(a.flow + 0, 1);
+    if (threadIdx.x == 0) *task_s = atomicAdd(a.flow + 0, 1);
     __syncthreads();
     for (;;) {
         const int t = *task_s;
@@ -455,45 +492,71 @@ __global__ void __launch_bounds__(NT, NT == 96 ? (AB > 21 ? 2 : AB > 12 ? 3 : kF
                         st4[4 * c4] = t4.x; st4[4 * c4 + 1] = t4.y; st4[4 * c4 + 2] = t4.z; st4[4 * c4 + 3] = t4.w;
                     }
                 }
-                if constexpr (!SPLIT) {
-#pragma unroll
-                    for (int m = 0; m + 1 < M; m += 2) {
-                        const float2 r2 = __fmul2_rn(make_float2(s[m], s[m + 1]),
-                                                     make_float2(octant_sign<M>(m, fx, fy, fz),
-                                                                 octant_sign<M>(m + 1, fx, fy, fz)));
-                        s[m] = r2.x;
-                        s[m + 1] = r2.y;
-                    }
-                    if constexpr (M % 2 == 1) s[M - 1] *= octant_sign<M>(M - 1, fx, fy, fz);
-                }
                 // moments -> directions (split: the record already holds them)
                 float psi[AB];
                 if constexpr (SPLIT) {
 #pragma unroll
                     for (int q = 0; q < AB; ++q) psi[q] = s[q];
+                } else if constexpr (SWAP) {
+                    // even and odd functions of the source, with the octant's signs
+                    float ev[NE_], od[NO_ > 0 ? NO_ : 1];
+#pragma unroll
+                    for (int k = 0; k < flow_even1(M); ++k)
+                        ev[k] = s[pos_of_lm(flow_even_lm(k), M)] * sign_lm(flow_even_lm(k), fx, fy, fz);
+#pragma unroll
+                    for (int k = 0; k < flow_odd1(M); ++k)
+                        od[k] = s[pos_of_lm(flow_odd_lm(k), M)] * sign_lm(flow_odd_lm(k), fx, fy, fz);
+#pragma unroll
+                    for (int k = 0; k < flow_comb(AB, M); ++k) {
+                        const float sa = s[pos_of_lm(swap_a(k, M), M)];
+                        const float tb = s[pos_of_lm(swap_b(k, M), M)] * (swap_s(k) * sign_lm(swap_b(k, M), fx, fy, fz));
+                        ev[flow_even1(M) + k] = fmaf(sa, sign_lm(swap_a(k, M), fx, fy, fz), tb);
+                        od[flow_odd1(M) + k] = fmaf(sa, sign_lm(swap_a(k, M), fx, fy, fz), -tb);
+                    }
+                    // the plain functions' sources and their exchange
+                    constexpr int NPL = flow_plain(AB, M) / 2;
+                    float2 sxy[NPL > 0 ? NPL : 1], syx[NPL > 0 ? NPL : 1];
+#pragma unroll
+                    for (int k = 0; k < NPL; ++k) {
+                        sxy[k] = make_float2(s[pos_of_lm(flow_plain_lm(2 * k), M)] * sign_lm(flow_plain_lm(2 * k), fx, fy, fz),
+                                             s[pos_of_lm(flow_plain_lm(2 * k + 1), M)] * sign_lm(flow_plain_lm(2 * k + 1), fx, fy, fz));
+                        syx[k] = make_float2(flow_plain_s(2 * k) * sxy[k].y, flow_plain_s(2 * k) * sxy[k].x);
+                    }
+                    // a pair's fluxes from its even and odd sums (two functions per packed
+                    // operation), a single direction's from the even one
+#pragma unroll
+                    for (int p = 0; p < NPR; ++p) {
+                        const float2 e = dot2<NE_>(dt.mop + flow_mop_pair(p, AB, M), ev);
+                        float2 t1 = e, t2 = e;
+                        if constexpr (NO_ > 0) {
+                            const float2 o1 = dot2<NO_>(dt.mop + flow_mop_odd(p, AB, M), od);
+                            t1 = __fadd2_rn(e, o1);
+                            t2 = __fadd2_rn(e, make_float2(-o1.x, -o1.y));
+                        }
+#pragma unroll
+                        for (int k = 0; k < NPL; ++k) {
+                            const float2 c1 = make_float2(dt.mop[flow_mop_pair_pl(p, AB, M) + 2 * k],
+                                                          dt.mop[flow_mop_pair_pl(p, AB, M) + 2 * k + 1]);
+                            t1 = __ffma2_rn(c1, sxy[k], t1);
+                            t2 = __ffma2_rn(c1, syx[k], t2);
+                        }
+                        psi[p] = t1.x + t1.y;
+                        psi[NPR + p] = t2.x + t2.y;
+                    }
+#pragma unroll
+                    for (int f = 0; f < AB - 2 * NPR; ++f) {
+                        float2 t = dot2<NE_>(dt.mop + flow_mop_single(f, AB, M), ev);
+#pragma unroll
+                        for (int k = 0; k < NPL; ++k)
+                            t = __ffma2_rn(make_float2(dt.mop[flow_mop_single_pl(f, AB, M) + 2 * k],
+                                                       dt.mop[flow_mop_single_pl(f, AB, M) + 2 * k + 1]), sxy[k], t);
+                        psi[2 * NPR + f] = t.x + t.y;
+                    }
                 } else {
-                    // even and odd moments in the two lanes of packed FMAs; the lane
-                    // sums of directions q, q+1 in one packed add
-                    auto msum = [&](int q) {
-                        float2 t2 = make_float2(0.0f, 0.0f);
 #pragma unroll
-                        for (int m = 0; m + 1 < M; m += 2)
-                            t2 = __ffma2_rn(make_float2(dt.mop[q * 16 + m], dt.mop[q * 16 + m + 1]),
-                                            make_float2(s[m], s[m + 1]), t2);
-                        if constexpr (M % 2 == 1) t2.x = fmaf(dt.mop[q * 16 + M - 1], s[M - 1], t2.x);
-                        return t2;
-                    };
+                    for (int m = 0; m < M; ++m) s[m] *= octant_sign<M>(m, fx, fy, fz);
 #pragma unroll
-                    for (int q = 0; q + 1 < AB; q += 2) {
-                        const float2 ta = msum(q), tb = msum(q + 1);
-                        const float2 p2 = __fadd2_rn(make_float2(ta.x, tb.x), make_float2(ta.y, tb.y));
-                        psi[q] = p2.x;
-                        psi[q + 1] = p2.y;
-                    }
-                    if constexpr (AB % 2 == 1) {
-                        const float2 ta = msum(AB - 1);
-                        psi[AB - 1] = ta.x + ta.y;
-                    }
+                    for (int q = 0; q < AB; ++q) psi[q] = dot<M>(dt.mop + q * 16, s);
                 }
                 // cell solve, PW directions at a time (the plane records' vector width)
                 const float* pv = buf + pb * P * RS;
@@ -600,31 +663,43 @@ __global__ void __launch_bounds__(NT, NT == 96 ? (AB > 21 ? 2 : AB > 12 ? 3 : kF
                     store_record<AB>(momg + (size_t)v * ABP, psi);
                 } else {
                     // directions -> moments (Eq. 3 for lm = 00): table rows hold w R_lm
-                    // even and odd directions in the two lanes of packed FMAs
                     float acc[M];
-                    // sum over directions of moment m, even and odd directions in the two lanes
-                    auto dsum = [&](int m) {
-                        float2 t2 = make_float2(0.0f, 0.0f);
+                    if constexpr (SWAP) {
 #pragma unroll
-                        for (int q = 0; q + 1 < AB; q += 2)
-                            t2 = __ffma2_rn(make_float2(dt.dop[m * kFlowMaxAB + q], dt.dop[m * kFlowMaxAB + q + 1]),
-                                            make_float2(psi[q], psi[q + 1]), t2);
-                        if constexpr (AB % 2 == 1) t2.x = fmaf(dt.dop[m * kFlowMaxAB + AB - 1], psi[AB - 1], t2.x);
-                        return t2;
-                    };
+                        for (int k = 0; k < flow_plain(AB, M); ++k)
+                            acc[pos_of_lm(flow_plain_lm(k), M)] =
+                                dot<AB>(dt.dop + flow_dop_plain(k, AB, M), psi) * sign_lm(flow_plain_lm(k), fx, fy, fz);
+                        // sums (and the single directions) and differences of the pairs
+                        float es[AB - NPR], fs[NPR > 0 ? NPR : 1];
 #pragma unroll
-                    for (int m = 0; m + 1 < M; m += 2) {
-                        // lane sums and octant signs of moments m, m+1 in one packed add and multiply
-                        const float2 ta = dsum(m), tb = dsum(m + 1);
-                        const float2 r2 = __fmul2_rn(__fadd2_rn(make_float2(ta.x, tb.x), make_float2(ta.y, tb.y)),
-                                                     make_float2(octant_sign<M>(m, fx, fy, fz),
-                                                                 octant_sign<M>(m + 1, fx, fy, fz)));
-                        acc[m] = r2.x;
-                        acc[m + 1] = r2.y;
-                    }
-                    if constexpr (M % 2 == 1) {
-                        const float2 ta = dsum(M - 1);
-                        acc[M - 1] = (ta.x + ta.y) * octant_sign<M>(M - 1, fx, fy, fz);
+                        for (int p = 0; p < NPR; ++p) {
+                            es[p] = psi[p] + psi[NPR + p];
+                            fs[p] = psi[p] - psi[NPR + p];
+                        }
+#pragma unroll
+                        for (int f = 0; f < AB - 2 * NPR; ++f) es[NPR + f] = psi[2 * NPR + f];
+#pragma unroll
+                        for (int k = 0; k < flow_even1(M); ++k)
+                            acc[pos_of_lm(flow_even_lm(k), M)] =
+                                dot<AB - NPR>(dt.dop + flow_dop_even(k, AB), es) * sign_lm(flow_even_lm(k), fx, fy, fz);
+#pragma unroll
+                        for (int k = 0; k < flow_odd1(M); ++k) {
+                            float t = 0.0f;
+                            if constexpr (NPR > 0) t = dot<NPR>(dt.dop + flow_dop_odd(k, AB, M), fs);
+                            acc[pos_of_lm(flow_odd_lm(k), M)] = t * sign_lm(flow_odd_lm(k), fx, fy, fz);
+                        }
+#pragma unroll
+                        for (int k = 0; k < flow_comb(AB, M); ++k) {
+                            const float e = dot<AB - NPR>(dt.dop + flow_dop_even(flow_even1(M) + k, AB), es);
+                            float o1 = 0.0f;
+                            if constexpr (NPR > 0) o1 = dot<NPR>(dt.dop + flow_dop_odd(flow_odd1(M) + k, AB, M), fs);
+                            acc[pos_of_lm(swap_a(k, M), M)] = (e + o1) * sign_lm(swap_a(k, M), fx, fy, fz);
+                            acc[pos_of_lm(swap_b(k, M), M)] = (e - o1) * (swap_s(k) * sign_lm(swap_b(k, M), fx, fy, fz));
+                        }
+                    } else {
+#pragma unroll
+                        for (int m = 0; m < M; ++m)
+                            acc[m] = dot<AB>(dt.dop + m * kFlowMaxAB, psi) * octant_sign<M>(m, fx, fy, fz);
                     }
                     if constexpr (COOP) {
                         // into the consumed source slot, from where four lanes reduce each record
@@ -668,10 +743,10 @@ __global__ void __launch_bounds__(NT, NT == 96 ? (AB > 21 ? 2 : AB > 12 ? 3 : kF
         }
     }
     __syncthreads();
-    for (int e = tid; e < gcount; e += blockDim.x)
+    for (int e = threadIdx.x; e < gcount; e += blockDim.x)
         if (leak_s[e] != 0.0) atomicAdd(a.leak + g0 + e, leak_s[e]);
     // the last CTA out resets the queue for the next sweep
-    if (tid == 0) {
+    if (threadIdx.x == 0) {
         __threadfence();
         if (atomicAdd(a.flow + 1, 1) == (int)gridDim.x - 1) {
             a.flow[0] = 0;
