@@ -175,7 +175,7 @@ ChainDirTable make_swap_table(const doctors_problem* p) {
 void free_problem(doctors_problem* p) {
     void* ptrs[] = {p->d_coef, p->d_mat, p->d_rho, p->d_sigt, p->d_sigs,
                     p->d_phiu_src, p->d_phiu, p->d_U, p->d_Q, p->d_mom, p->d_src, p->d_src2, p->d_prev,
-                    p->d_emit, p->d_iso, p->d_xface, p->d_yface, p->d_red,
+                    p->d_emit, p->d_raysrc, p->d_iso, p->d_xface, p->d_yface, p->d_red,
                     p->d_Z, p->d_Qa, p->d_T, p->d_rf, p->d_r, p->d_acc, p->d_grad, p->d_H,
                     p->d_ones, p->d_psi, p->d_prod, p->d_flow, p->d_qang, p->d_pang,
                     p->d_k, p->d_roi, p->d_part, p->d_tcb, p->d_emit_all, p->d_dose_stage, p->d_sig};
@@ -235,11 +235,13 @@ int check_problem(doctors_problem* p) {
 // ray trace every point source and build the fixed (first-collision) source Q
 int first_collision(doctors_problem* p) {
     const size_t GV = (size_t)p->G * p->V;
-    CU(cudaMemsetAsync(p->d_phiu, 0, GV * sizeof(float), p->stream));
-    // the first point source stores the uncollided moments, later ones add;
-    // with volume sources only they stay zero
     bool any_point = false;
     for (const doctors_source& src : p->srcs) any_point = any_point || src.kind != DOCTORS_SRC_VOLUME;
+    // sources are traced in chunks: their path lengths per material go through the
+    // sweep source's buffer (free before the iteration); where not one source's fit
+    // (more materials than groups x moments), source by source
+    const size_t chunk = (size_t)p->G * p->M / p->nmat;
+    if (!any_point || chunk == 0) CU(cudaMemsetAsync(p->d_phiu, 0, GV * sizeof(float), p->stream));
     if (!any_point) CU(cudaMemsetAsync(p->d_U, 0, GV * p->M * sizeof(float), p->stream));
     bool first_point = true;
     std::vector<float> iso(p->G, 0.0f);
@@ -263,12 +265,43 @@ int first_collision(doctors_problem* p) {
     float* d_emit_all = p->d_emit_all;
     cudaError_t e = cudaMemcpyAsync(d_emit_all, emit_all.data(), emit_all.size() * sizeof(float),
                                     cudaMemcpyHostToDevice, p->stream);
-    for (size_t s = 0; s < p->srcs.size() && e == cudaSuccess; ++s) {
+    std::vector<RaySource> points;
+    for (size_t s = 0; s < p->srcs.size(); ++s) {
         const doctors_source& src = p->srcs[s];
         if (src.kind == DOCTORS_SRC_VOLUME) {
             for (int g = 0; g < p->G; ++g) iso[g] += (float)(src.weight * p->spectra[s][g]);
             continue;
         }
+        const RayArgs r = ray_args(p, src, nullptr);
+        points.push_back({r.sx, r.sy, r.sz, r.ax, r.ay, r.az, r.px, r.py, r.pz, r.ux, r.uy, r.uz, r.tan_half, r.z_slope,
+                          r.lit_all, (int)s});
+    }
+    if (chunk > 0 && !points.empty()) {
+        if (p->raysrc_cap < points.size()) {
+            if (p->d_raysrc) {
+                CU(cudaStreamSynchronize(p->stream));
+                cudaFree(p->d_raysrc);
+                p->d_raysrc = nullptr;
+                p->raysrc_cap = 0;
+            }
+            int rc = dalloc_t(&p->d_raysrc, points.size(), "source geometry");
+            if (rc) return rc;
+            p->raysrc_cap = points.size();
+        }
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(p->d_raysrc, points.data(), points.size() * sizeof(RaySource), cudaMemcpyHostToDevice, p->stream);
+        const RayArgs r = ray_args(p, p->srcs[points[0].row], d_emit_all);
+        // one launch's grid holds at most 65535 sources, far above the source limit
+        for (size_t c = 0; c < points.size() && e == cudaSuccess; c += chunk) {
+            const int n = (int)std::min(chunk, points.size() - c);
+            e = launch_ray_lengths(r, p->d_raysrc + c, n, p->d_src, p->stream);
+            if (e == cudaSuccess) e = launch_uncollided(r, p->d_raysrc + c, n, p->d_src, p->d_U, p->M, c == 0, p->stream);
+            p->launches += 2;
+        }
+    }
+    for (size_t s = 0; chunk == 0 && s < p->srcs.size() && e == cudaSuccess; ++s) {
+        const doctors_source& src = p->srcs[s];
+        if (src.kind == DOCTORS_SRC_VOLUME) continue;
         RayArgs r = ray_args(p, src, d_emit_all + s * p->G);
         e = launch_raytrace(r, p->stream);
         if (e != cudaSuccess) break;

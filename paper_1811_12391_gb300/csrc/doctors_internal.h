@@ -48,7 +48,21 @@ struct RayArgs {
     float* phi_tot;                    // [G][V] accumulated (+=), or null
 };
 
+// One point source of a chunk traced together (fields as RayArgs); row: its row
+// of the emission table a.emit [..][G]
+struct RaySource {
+    float sx, sy, sz, ax, ay, az, px, py, pz, ux, uy, uz, tan_half, z_slope;
+    int lit_all, row;
+};
+
 cudaError_t launch_raytrace(const RayArgs& a, cudaStream_t s);
+// density-weighted path lengths per material of n sources: lam [n][nmat][V]
+// (unlit voxels are not written)
+cudaError_t launch_ray_lengths(const RayArgs& a, const RaySource* src, int n, float* lam, cudaStream_t s);
+// their uncollided fluence into a.phi_tot and its moments into U [G][V][M]:
+// stored (first) or added
+cudaError_t launch_uncollided(const RayArgs& a, const RaySource* src, int n, const float* lam, float* U, int M, bool first,
+                              cudaStream_t s);
 cudaError_t launch_debug_ray(const RayArgs& a, int voxel, int32_t* idx, float* len, int cap,
                              int* count, cudaStream_t s);
 cudaError_t launch_backproject(const RayArgs& a, const float* H, double* grad, cudaStream_t s);
@@ -484,6 +498,8 @@ struct doctors_problem {
     float* d_emit = nullptr;       // [G]
     float* d_emit_all = nullptr;   // [n_src][G] weight * spectrum of every source
     size_t emit_cap = 0;           // floats allocated in d_emit_all
+    doctors::RaySource* d_raysrc = nullptr;   // [n_src] geometry of the point sources
+    size_t raysrc_cap = 0;
     float* d_iso = nullptr;        // [G]
     float* d_xface = nullptr;
     float* d_yface = nullptr;
