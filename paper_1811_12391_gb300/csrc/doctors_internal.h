@@ -202,7 +202,7 @@ struct SweepArgs {
     float* yface;                      // [8][A8][G][nty-1][nx][nz]
     double* leak;                      // [G]
     int A;                             // directions (psi indexing)
-    float* psi;                        // written (mode 1) or read (mode 2): [G][V][A], dataflow kernel [G][V][8][ABP]
+    float* psi;                        // written (mode 1) or read (mode 2): [G][V][A], dataflow kernel [G][8][V][nab][ABP]
     float* prod;                       // [G][V]: mode 2 accumulator
     const int* skip;                   // if non-null and *skip != 0 the kernel does nothing
     int depth;                         // dataflow kernels: steps of source and face records held in shared memory

@@ -485,7 +485,7 @@ __global__ void __launch_bounds__(NT, NT == 96 ? (AB > 12 ? 4 : kFlowMinCtas) : 
                 float st4[MODE == 2 ? ABP : 1];     // stored angular fluence (mode 2), read ahead of its use
                 if constexpr (MODE == 2) {
                     const float4* rec =
-                        reinterpret_cast<const float4*>(a.psi + ((((size_t)g * V + v) * 8 + oe) * a.nab + a.blk) * ABP);
+                        reinterpret_cast<const float4*>(a.psi + ((ang0 + v) * a.nab + a.blk) * ABP);
 #pragma unroll
                     for (int c4 = 0; c4 < ABP / 4; ++c4) {
                         const float4 t4 = __ldg(rec + c4);
@@ -610,10 +610,13 @@ __global__ void __launch_bounds__(NT, NT == 96 ? (AB > 12 ? 4 : kFlowMinCtas) : 
                     if constexpr (DD) plane_store_w<PW>(cvy + os + q0, py);
                 }
                 // stored angular fluence, laid out for this kernel as one 16-byte
-                // aligned record of ABP floats per (group, voxel, direction octant,
-                // direction block): [G][V][8][nab][ABP] (the stage kernels use [G][V][A])
+                // aligned record of ABP floats per (group, direction octant, voxel,
+                // direction block): [G][8][V][nab][ABP] (the stage kernels use [G][V][A]).
+                // A record need not fill its last 32-byte sector; this way the x
+                // neighbour, one step later, fills it while it is still in L2 (with the
+                // octants of a voxel side by side it was written back half full)
                 if constexpr (MODE == 1)
-                    store_record<AB>(a.psi + ((((size_t)g * V + v) * 8 + oe) * a.nab + a.blk) * ABP, psi);
+                    store_record<AB>(a.psi + ((ang0 + v) * a.nab + a.blk) * ABP, psi);
                 if constexpr (MODE == 2) {
                     float pacc = 0.0f;
 #pragma unroll
