@@ -338,6 +338,22 @@ __global__ void __launch_bounds__(kScatterThreads, GMAX <= 24 ? 2 : 1) k_scatter
     }
 }
 
+// The adjoint's fixed source: scale * field in the l = 0 moment, nothing else
+// (one 16-byte store per thread and pass; M = 1, 9: one entry).  Floor: the
+// moments written once, 25 us at 19 groups x 64x64x32, P3; the general kernel,
+// which loops over groups per entry, takes 231 us.
+template <int VEC>
+__global__ void __launch_bounds__(256) k_iso_source(size_t GV, int M, const float* field, float scale, float* out) {
+    const unsigned per = (unsigned)M / VEC;              // vectors per record
+    const size_t n = GV * per;
+    for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
+        const size_t e = t / per;
+        const float x = t - e * per == 0 ? scale * __ldg(field + e) : 0.0f;
+        if constexpr (VEC == 4) reinterpret_cast<float4*>(out)[t] = make_float4(x, 0.0f, 0.0f, 0.0f);
+        else out[t] = x;
+    }
+}
+
 template <int NV>
 __device__ __forceinline__ void block_reduce_add(double (&x)[NV], double* dst) {
     __shared__ double red[NV][32];
@@ -556,6 +572,14 @@ cudaError_t launch_scatter_g(const ScatterArgs& a, cudaStream_t s) {
 }
 
 cudaError_t launch_scatter(const ScatterArgs& a, cudaStream_t s) {
+    if (!a.phi && !a.base && !a.iso && a.iso_field && !a.skip && !a.win && a.g0 == 0 && (a.g1 == 0 || a.g1 == a.G)) {
+        const size_t GV = (size_t)a.G * a.V;
+        if (a.M % 4 == 0)
+            k_iso_source<4><<<blocks_for(GV * a.M / 4, 256, 152 * 16), 256, 0, s>>>(GV, a.M, a.iso_field, a.iso_field_scale, a.out);
+        else
+            k_iso_source<1><<<blocks_for(GV * a.M, 256, 152 * 16), 256, 0, s>>>(GV, a.M, a.iso_field, a.iso_field_scale, a.out);
+        return cudaGetLastError();
+    }
     if (a.G <= 8) return launch_scatter_g<8>(a, s);
     if (a.G <= 16) return launch_scatter_g<16>(a, s);
     if (a.G <= 20) return launch_scatter_g<20>(a, s);
