@@ -88,8 +88,9 @@ typedef struct doctors_options {
     double tol;              /* stop when, in every group, ||phi00_new - phi00_old||_2 / ||phi00_new||_2 < tol;
                                 values below 1e-6 are raised to 1e-6 (FP32 sweep) */
     int max_iters;           /* source-iteration cap, >= 1 */
-    int tile_x, tile_y;      /* sweep tile in voxels (0 = default: 8 x 8 for the dataflow sweep, else
-                                16 x 16); tile_x*tile_y <= 256 */
+    int tile_x, tile_y;      /* sweep tile in voxels (0 = default: 8 x 8 for the dataflow sweep, 16 x 16
+                                for its P0 and P1 sweeps up to S8 on most meshes and for the other
+                                kernels); tile_x*tile_y <= 256 */
     int angles_per_block;    /* directions per sweep block (0 = default: whole octants on the dataflow
                                 sweep, else the largest of 12, 10, 9, 7, ... dividing it); must divide
                                 N(N+2)/8; 21 and 36 (whole S12, S16 octants) on the dataflow sweep only */

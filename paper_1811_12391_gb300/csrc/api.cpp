@@ -954,7 +954,22 @@ int doctors_create_problem(const doctors_mesh* mesh, const doctors_options* opt,
     // measured shapes)
     const bool flow_default = opt->sweep_kernel >= 4 || p->differencing == DOCTORS_DIFF_DIAMOND ||
                               (opt->sweep_kernel == 0 && kDefaultDataflowSweep && flow_block_ab(p->A8, p->ab));
-    const int tdef = flow_default ? 8 : 16;
+    // With P0 and P1 up to S8 a cell step is short, and handing faces from tile to
+    // tile costs more than the longer fill of a 16 x 16 tile, unless its ragged
+    // edge sweeps many more columns (8 x 8 -> 16 x 16, ms per sweep: 64x64x16 S6 P0
+    // 0.106 -> 0.094, S8 P1 0.153 -> 0.140, 256x256x64 S6 P0 3.03 -> 2.79, 75x61x37
+    // S4 P1 0.260 -> 0.236, 20x150x12 S6 P0 0.122 -> 0.108; but 40x33x20, where it
+    // sweeps 1.44 times the columns, S6 P1 0.077 -> 0.083; with P3 64x64x32 S8 0.63
+    // -> 0.78, with S12 and S16 1.2 to 1.4 times slower)
+    int tdef = flow_default ? 8 : 16;
+    if (flow_default && p->A8 == p->ab && p->M <= 4 && p->ab <= 10 && opt->tile_x <= 0 && opt->tile_y <= 0) {
+        auto columns = [&](int t) {
+            const int tx = std::min(t, p->nx), ty = std::min(t, p->ny);
+            return (double)((p->nx + tx - 1) / tx * tx) * ((p->ny + ty - 1) / ty * ty);
+        };
+        const double ratio = columns(16) / columns(8);
+        if (ratio <= 1.25 || (ratio <= 1.5 && std::max(p->nx, p->ny) >= 96)) tdef = 16;
+    }
     p->tx = opt->tile_x > 0 ? opt->tile_x : std::min(tdef, p->nx);
     p->ty = opt->tile_y > 0 ? opt->tile_y : std::min(tdef, p->ny);
     auto fail = [&](int code, const std::string& msg) {
@@ -1494,7 +1509,7 @@ int ensure_adjoint_buffers(doctors_problem* p, bool density) {
     if (!p->d_grad) rc = rc ? rc : dalloc_t(&p->d_grad, p->V, "density gradient");
     if (density) {
         if (!p->d_H) rc = rc ? rc : dalloc_t(&p->d_H, (size_t)kMaxMat * p->V, "ray importance");
-        // [G][V][A] for the stage kernels, [G][V][8][A/8 padded to 4] for the dataflow kernel
+        // [G][V][A] for the stage kernels, [G][8][V][A/8 padded to 4] for the dataflow kernel
         if (!p->d_psi)
             rc = rc ? rc : dalloc_t(&p->d_psi, GV * std::max((size_t)p->A, (size_t)8 * flow_abp_host(p->A8)),
                                     "stored angular fluence");
