@@ -430,14 +430,9 @@ int iterate(doctors_problem* p, int reverse, const float* Q, float* mom, doctors
     // tol and whose sources are all final is final itself: in the forward
     // problem (downscatter) the window's leading groups retire, in the adjoint
     // (transposed scattering, upward in energy) its trailing groups.
-    int g0 = 0, g1 = p->G;
-    std::vector<double> eps(p->G, 0.0);
-    // The next iteration's scattering source is formed while the host reads
-    // this iteration's residuals: it is launched right after the residual
-    // copy, for the current window (a superset of the next one), into the
-    // other source buffer; the host waits only for the copy.  After the last
-    // iteration that launch is wasted, and the source of the last sweep stays
-    // in its own buffer for the balance.
+    // The next iteration's scattering source is formed for the window just swept
+    // (a superset of the next one) into the other source buffer, so the source of
+    // the last sweep stays in its own buffer for the balance.
     float* srcs[2] = {p->d_src, p->d_src2};
     int cur = 0;
     SweepArgs sw = sweep_args(p, reverse, srcs[cur], mom);
@@ -446,60 +441,130 @@ int iterate(doctors_problem* p, int reverse, const float* Q, float* mom, doctors
     sa.mat = p->d_mat; sa.rho = p->d_rho; sa.sigs = p->d_sigs;
     sa.base = Q; sa.phi = mom;
     CU(cudaMemcpyAsync(srcs[cur], Q, GVM * sizeof(float), cudaMemcpyDeviceToDevice, p->stream));
-    while (it < p->opt.max_iters) {
-        const int gc = g1 - g0;
-        if (!p->use_split)   // the split path's d2m pass writes the window's moments
-            CU(cudaMemsetAsync(mom + (size_t)g0 * VM, 0, (size_t)gc * VM * sizeof(float), p->stream));
-        CU(cudaMemsetAsync(p->d_red + g0, 0, (size_t)gc * sizeof(double), p->stream));
-        CU(cudaMemsetAsync(d_res + 2 * g0, 0, 2 * (size_t)gc * sizeof(double), p->stream));
-        CU(cudaEventRecord(p->ev[3], p->stream));
-        sw.src = srcs[cur];
-        sw.g0 = g0;
-        sw.gcount = gc;
-        int nl = 0;
-        CU(launch_sweep(p, sw, 0, p->stream, &nl));
-        p->launches += nl;
-        CU(cudaEventRecord(p->ev[4], p->stream));
-        CU(launch_residual(p->V, p->G, p->M, mom, p->d_prev, d_res, p->stream, nullptr, g0, gc));
-        ++p->launches;
-        CU(cudaMemcpyAsync(p->h_red, p->d_red, 3 * (size_t)p->G * sizeof(double), cudaMemcpyDeviceToHost,
-                           p->stream));
-        CU(cudaEventRecord(p->ev[5], p->stream));
-        const bool ahead = it + 1 < p->opt.max_iters;
-        if (ahead) {
-            sa.g0 = g0;
-            sa.g1 = g1;
-            sa.out = srcs[cur ^ 1];
-            CU(launch_scatter(sa, p->stream));
-            ++p->launches;
-        }
-        CU(cudaEventSynchronize(p->ev[5]));
-        float ms = 0.0f;
-        CU(cudaEventElapsedTime(&ms, p->ev[3], p->ev[4]));
-        ms_sweep += ms;
-        updates += (double)p->V * p->A * gc;
-        ++it;
-        resid = 0.0;
-        for (int g = g0; g < g1; ++g) {
-            const double num = p->h_red[p->G + 2 * g], den = p->h_red[p->G + 2 * g + 1];
-            eps[g] = den > 0.0 ? std::sqrt(num / den) : 0.0;
-            if (!std::isfinite(eps[g])) {
-                CU(cudaStreamSynchronize(p->stream));
-                set_error("source iteration produced a non-finite fluence");
-                return DOCTORS_ERR_INVALID_ARG;
+    if (p->use_flow) {
+        // The dataflow sweep and the kernels around it read the window and whether
+        // the loop has ended from device memory, so the host enqueues an iteration
+        // before it knows how the one before it ended, and the GPU never waits for
+        // the host; what it enqueued past the end does nothing.  (Paper coarse
+        // mesh, S6 P0, 15 iterations: the GPU idled 45 us per iteration for the
+        // residual's round trip and eight launches.)
+        LoopCtl c{};
+        c.max_iters = p->opt.max_iters;
+        c.G = p->G;
+        c.tol = tol;
+        c.res = d_res;
+        c.reverse = reverse;
+        c.use_window = 1;
+        c.win[1] = p->G;
+        CU(cudaMemcpyAsync(p->d_ctl, &c, sizeof(c), cudaMemcpyHostToDevice, p->stream));
+        sw.skip = sa.skip = &p->d_ctl->done;
+        sw.win = p->d_ctl->win;
+        sa.win = p->d_ctl->swept;
+        sa.zero_mom = mom;
+        sa.zero_win = p->d_ctl->win;
+        sa.zero_red = p->d_red;
+        auto enqueue = [&](int i) -> int {
+            cudaEvent_t* ev = p->ev + 3 + 3 * (i & 1);
+            CU(cudaEventRecord(ev[0], p->stream));
+            sw.src = srcs[i & 1];
+            int nl = 0;
+            CU(launch_sweep(p, sw, 0, p->stream, &nl));
+            CU(cudaEventRecord(ev[1], p->stream));
+            CU(launch_residual(p->V, p->G, p->M, mom, p->d_prev, d_res, p->stream, sw.skip, 0, -1, sw.win, p->d_ctl,
+                               p->h_ctl + (i & 1)));
+            CU(cudaEventRecord(ev[2], p->stream));
+            if (i + 1 < p->opt.max_iters) {
+                sa.out = srcs[(i + 1) & 1];
+                CU(launch_scatter(sa, p->stream));
+                ++p->launches;
             }
-            resid = std::max(resid, eps[g]);
+            p->launches += nl + 1;
+            return DOCTORS_OK;
+        };
+        int rc = enqueue(0);
+        if (rc) return rc;
+        for (int i = 0;; ++i) {
+            if (i + 1 < p->opt.max_iters) {
+                rc = enqueue(i + 1);
+                if (rc) return rc;
+            }
+            cudaEvent_t* ev = p->ev + 3 + 3 * (i & 1);
+            CU(cudaEventSynchronize(ev[2]));
+            float ms = 0.0f;
+            CU(cudaEventElapsedTime(&ms, ev[0], ev[1]));
+            ms_sweep += ms;
+            c = p->h_ctl[i & 1];
+            if (c.done) break;
         }
-        if (resid < tol) {
-            conv = true;
-            break;
+        it = c.iters;
+        resid = c.resid;
+        updates = (double)c.group_sweeps * (double)p->V * p->A;
+        cur = (it - 1) & 1;
+        if (!std::isfinite(resid)) {
+            CU(cudaStreamSynchronize(p->stream));
+            set_error("source iteration produced a non-finite fluence");
+            return DOCTORS_ERR_INVALID_ARG;
         }
-        if (!ahead) break;
-        if (!reverse)
-            while (g0 < g1 - 1 && eps[g0] < tol) ++g0;
-        else
-            while (g1 - 1 > g0 && eps[g1 - 1] < tol) --g1;
-        cur ^= 1;
+        conv = resid < tol;
+    } else {
+        // the other sweep kernels: the host reads the residuals and sets the window
+        int g0 = 0, g1 = p->G;
+        std::vector<double> eps(p->G, 0.0);
+        while (it < p->opt.max_iters) {
+            const int gc = g1 - g0;
+            if (!p->use_split)   // the split path's d2m pass writes the window's moments
+                CU(cudaMemsetAsync(mom + (size_t)g0 * VM, 0, (size_t)gc * VM * sizeof(float), p->stream));
+            CU(cudaMemsetAsync(p->d_red + g0, 0, (size_t)gc * sizeof(double), p->stream));
+            CU(cudaMemsetAsync(d_res + 2 * g0, 0, 2 * (size_t)gc * sizeof(double), p->stream));
+            CU(cudaEventRecord(p->ev[3], p->stream));
+            sw.src = srcs[cur];
+            sw.g0 = g0;
+            sw.gcount = gc;
+            int nl = 0;
+            CU(launch_sweep(p, sw, 0, p->stream, &nl));
+            p->launches += nl;
+            CU(cudaEventRecord(p->ev[4], p->stream));
+            CU(launch_residual(p->V, p->G, p->M, mom, p->d_prev, d_res, p->stream, nullptr, g0, gc));
+            ++p->launches;
+            CU(cudaMemcpyAsync(p->h_red, p->d_red, 3 * (size_t)p->G * sizeof(double), cudaMemcpyDeviceToHost,
+                               p->stream));
+            CU(cudaEventRecord(p->ev[5], p->stream));
+            const bool ahead = it + 1 < p->opt.max_iters;
+            if (ahead) {
+                sa.g0 = g0;
+                sa.g1 = g1;
+                sa.out = srcs[cur ^ 1];
+                CU(launch_scatter(sa, p->stream));
+                ++p->launches;
+            }
+            CU(cudaEventSynchronize(p->ev[5]));
+            float ms = 0.0f;
+            CU(cudaEventElapsedTime(&ms, p->ev[3], p->ev[4]));
+            ms_sweep += ms;
+            updates += (double)p->V * p->A * gc;
+            ++it;
+            resid = 0.0;
+            for (int g = g0; g < g1; ++g) {
+                const double num = p->h_red[p->G + 2 * g], den = p->h_red[p->G + 2 * g + 1];
+                eps[g] = den > 0.0 ? std::sqrt(num / den) : 0.0;
+                if (!std::isfinite(eps[g])) {
+                    CU(cudaStreamSynchronize(p->stream));
+                    set_error("source iteration produced a non-finite fluence");
+                    return DOCTORS_ERR_INVALID_ARG;
+                }
+                resid = std::max(resid, eps[g]);
+            }
+            if (resid < tol) {
+                conv = true;
+                break;
+            }
+            if (!ahead) break;
+            if (!reverse)
+                while (g0 < g1 - 1 && eps[g0] < tol) ++g0;
+            else
+                while (g1 - 1 > g0 && eps[g1 - 1] < tol) --g1;
+            cur ^= 1;
+        }
     }
     // particle balance of the last sweep (FP64)
     const double vol = p->mesh.dx * p->mesh.dy * p->mesh.dz;
@@ -782,17 +847,28 @@ int configure_sweep(doctors_problem* p, int tx, int ty, int ab, int kernel) {
         // with four) or does not fit at all
         const int threads = flow_threads(tx, ty);
         int per_sm = 0, per_sm_main = 0;
-        for (int depth = 2; depth <= 4; depth += 2) {
-            const size_t sf = sweep_flow_smem_bytes(ab, p->M, tx, ty, p->G, depth, dd);
-            const size_t ss = use_split ? sweep_flow_smem_bytes(ab, flow_abp_host(ab), tx, ty, p->G, depth) : 0;
-            if (depth == 2) smem = std::max(sf, ss);
-            if (std::max(sf, ss) > 227 * 1024) break;
-            const int b = sweep_flow_blocks_per_sm(ab, p->M, threads, sf, false, dd);
-            const int bm = use_split ? sweep_flow_blocks_per_sm(ab, p->M, threads, ss, true) : b;
-            if (depth == 2 || (b >= per_sm && bm >= per_sm_main)) {
+        const int rf_split = flow_abp_host(ab);
+        auto fused = [&](int depth) { return sweep_flow_smem_bytes(ab, p->M, tx, ty, p->G, depth, dd); };
+        auto split = [&](int depth) { return use_split ? sweep_flow_smem_bytes(ab, rf_split, tx, ty, p->G, depth) : (size_t)0; };
+        auto query = [&](int depth, int* b, int* bm) {
+            *b = sweep_flow_blocks_per_sm(ab, p->M, threads, fused(depth), false, dd);
+            *bm = use_split ? sweep_flow_blocks_per_sm(ab, p->M, threads, split(depth), true) : *b;
+        };
+        smem = std::max(fused(2), split(2));
+        if (std::max(fused(4), split(4)) <= 227 * 1024) {
+            query(4, &per_sm, &per_sm_main);
+            flow_depth = 4;
+        }
+        // shared memory of one more CTA left over: registers limit both depths alike
+        auto spare = [&](size_t bytes, int ctas) { return (size_t)(ctas + 1) * (bytes + 1024) <= 228 * 1024; };
+        if (smem <= 227 * 1024 &&
+            !(per_sm > 0 && per_sm_main > 0 && spare(fused(4), per_sm) && (!use_split || spare(split(4), per_sm_main)))) {
+            int b = 0, bm = 0;
+            query(2, &b, &bm);
+            if (b > per_sm || bm > per_sm_main) {
                 per_sm = b;
                 per_sm_main = bm;
-                flow_depth = depth;
+                flow_depth = 2;
             }
         }
         if (smem <= 227 * 1024) {
@@ -1057,10 +1133,13 @@ int doctors_create_problem(const doctors_mesh* mesh, const doctors_options* opt,
         if (p->dir_flow.w[0] <= 0.0f) return fail(DOCTORS_ERR_INVALID_ARG, "quadrature is not symmetric in x and y");
     }
     rc = rc ? rc : configure_sweep(p, p->tx, p->ty, p->ab, opt->sweep_kernel);
-    rc = rc ? rc : dalloc_t(&p->d_red, 5 * (size_t)p->G, "reductions");
+    static_assert(sizeof(LoopCtl) % sizeof(double) == 0, "loop state after the reductions");
+    rc = rc ? rc : dalloc(reinterpret_cast<void**>(&p->d_red), 5 * (size_t)p->G * sizeof(double) + sizeof(LoopCtl), "reductions");
     if (rc) return fail(rc, "");
-    e = cudaMallocHost(&p->h_red, 5 * (size_t)p->G * sizeof(double));
+    e = cudaMallocHost(&p->h_red, 5 * (size_t)p->G * sizeof(double) + 2 * sizeof(LoopCtl));
     if (e != cudaSuccess) return fail(DOCTORS_ERR_OOM, "pinned host allocation failed");
+    p->d_ctl = reinterpret_cast<LoopCtl*>(p->d_red + 5 * p->G);
+    p->h_ctl = reinterpret_cast<LoopCtl*>(p->h_red + 5 * p->G);
     for (auto& ev : p->ev) {
         e = cudaEventCreate(&ev);
         if (e != cudaSuccess) return fail(DOCTORS_ERR_CUDA, "cudaEventCreate failed");

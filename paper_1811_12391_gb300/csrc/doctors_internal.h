@@ -136,13 +136,16 @@ struct ScatterArgs {
     const int* skip;                   // if non-null and *skip != 0 the kernel does nothing
     int g0, g1;                        // destination groups updated: g0 .. g1 - 1 (g1 = 0: all)
     const int* win;                    // non-null: the window [win[0], win[1]) in device memory instead
+    float* zero_mom;                   // non-null (then phi itself): the groups of zero_win are zeroed once read,
+    const int* zero_win;               // with their leakage zero_red[g] and every residual sum
+    double* zero_red;                  // zero_red[G .. 3G)
 };
 cudaError_t launch_scatter(const ScatterArgs& a, cudaStream_t s);
 
 // residual: res[g][0] += sum_v (phi00 - prev)^2, res[g][1] += sum_v phi00^2; prev = phi00
 cudaError_t launch_residual(size_t V, int G, int M, const float* mom, float* prev, double* res,
                             cudaStream_t s, const int* skip = nullptr, int g0 = 0, int gcount = -1,
-                            const int* win = nullptr);
+                            const int* win = nullptr, struct LoopCtl* loop = nullptr, struct LoopCtl* host_copy = nullptr);
 // zero groups [win[0], win[1]) of a [G][per_group] float array unless *skip
 cudaError_t launch_zero_window(float* p, size_t per_group, int G, const int* win, const int* skip, cudaStream_t s);
 // out[g][v] = rho[v] * sigt[mat[v]][g] (FP32, the product the sweep forms)
@@ -165,11 +168,12 @@ struct LoopCtl {
     int reverse;                       // adjoint: the window's trailing groups retire
     int use_window;                    // the instance's kernels follow win (else all groups, every sweep)
     int win[2];                        // active group window [win[0], win[1])
+    int swept[2];                      // window of the last sweep
+    unsigned arrived, pad;             // blocks of the residual that are done
     long long group_sweeps;            // sum over iterations of the groups swept
 };
 // Retire converged instances; end the while loop when all are retired.
 cudaError_t launch_decide(LoopCtl* ctl, int n, unsigned long long cond_handle, cudaStream_t s);
-
 // balance: bal[g][0] += vol * sum s00, bal[g][1] += vol * sum sigma_t phi00
 cudaError_t launch_balance(size_t V, int G, int M, const uint8_t* mat, const float* rho,
                            const float* sigt, const float* src, const float* mom, double vol,
@@ -504,8 +508,10 @@ struct doctors_problem {
     float* d_xface = nullptr;
     float* d_yface = nullptr;
     size_t xface_bytes = 0, yface_bytes = 0;
-    double* d_red = nullptr;       // reductions: leak [G], res [G][2], bal [G][2]
-    double* h_red = nullptr;       // pinned mirror
+    double* d_red = nullptr;       // reductions: leak [G], res [G][2], bal [G][2], then the loop state
+    double* h_red = nullptr;       // pinned mirror, then the loop state after the last two iterations
+    doctors::LoopCtl* d_ctl = nullptr;     // (in d_red)
+    doctors::LoopCtl* h_ctl = nullptr;     // (in h_red) [2]
     // adjoint state (allocated on the first adjoint solve)
     float* d_Z = nullptr;          // [G][V][M] adjoint moments
     float* d_Qa = nullptr;         // [G][V][M] adjoint fixed source
@@ -530,6 +536,6 @@ struct doctors_problem {
     double* d_dose_stage = nullptr;  // [V] dose staging for host-memory output
     bool solved = false;
     bool adjoint_done = false;
-    cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+    cudaEvent_t ev[9] = {};        // the last six: start, end of the sweep and end, of two iterations in flight
     long long launches = 0;        // kernels launched by the current call
 };

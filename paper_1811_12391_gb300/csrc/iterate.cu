@@ -274,7 +274,7 @@ size_t scatter_fast_table_bytes(const ScatterArgs& a) {
     return (size_t)a.nmat * (a.L + 1) * scatter_fast_pitch<GMAX>() * sizeof(float);
 }
 
-template <int GMAX, bool TR, bool HAS_BASE, bool ISO = false>
+template <int GMAX, bool TR, bool HAS_BASE, bool ISO = false, bool ZERO = false>
 __global__ void __launch_bounds__(kScatterThreads, GMAX <= 24 ? 2 : 1) k_scatter_fast(const ScatterArgs a) {
     extern __shared__ float4 tab4_s[];
     float* tab_s = reinterpret_cast<float*>(tab4_s);
@@ -291,6 +291,11 @@ __global__ void __launch_bounds__(kScatterThreads, GMAX <= 24 ? 2 : 1) k_scatter
     __syncthreads();
     const unsigned VM = (unsigned)(a.V * a.M), M = (unsigned)a.M;
     const int g_beg = a.win ? a.win[0] : a.g0, g_end = a.win ? a.win[1] : (a.g1 > 0 ? a.g1 : G);
+    const int z_beg = ZERO ? a.zero_win[0] : 0, z_end = ZERO ? a.zero_win[1] : 0;
+    if (ZERO && blockIdx.x == 0) {
+        for (int g = threadIdx.x; g < 2 * G; g += blockDim.x) a.zero_red[G + g] = 0.0;
+        for (int g = z_beg + threadIdx.x; g < z_end; g += blockDim.x) a.zero_red[g] = 0.0;
+    }
     const int L1 = a.L + 1;
     // no barrier below: threads leave the grid-stride loop independently
     for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < VM; t += gridDim.x * blockDim.x) {
@@ -302,8 +307,16 @@ __global__ void __launch_bounds__(kScatterThreads, GMAX <= 24 ? 2 : 1) k_scatter
         const float* pp = a.phi + t;
 #pragma unroll
         for (int gp = 0; gp < GMAX; ++gp) {
-            const float x = __ldg(pp + (size_t)(gp < G ? gp : G - 1) * VM);
+            const float* pg = pp + (size_t)(gp < G ? gp : G - 1) * VM;
+            const float x = ZERO ? *pg : __ldg(pg);
             ph[gp] = gp < G ? x : 0.0f;
+        }
+        if (ZERO) {
+            // read by no other thread: ready for the next sweep to add to
+            float* pz = a.zero_mom + t;
+#pragma unroll
+            for (int gp = 0; gp < GMAX; ++gp)
+                if (gp >= z_beg && gp < z_end) pz[(size_t)gp * VM] = 0.0f;
         }
         float qb[GMAX];
         const float* pb = a.base + t;
@@ -335,6 +348,54 @@ __global__ void __launch_bounds__(kScatterThreads, GMAX <= 24 ? 2 : 1) k_scatter
             const float out = fmaf(r, acc, qb[g]);
             if (g >= g_beg && g < g_end) po[(size_t)g * VM] = out;
         }
+    }
+}
+
+// Update a live instance's iteration count and residual (max over groups of
+// sqrt(sum (dphi)^2 / sum phi^2)), retire it when the relative change is below
+// its tolerance or the cap is reached, else shrink its active group window: a
+// group whose relative change is below tol and whose sources are all final is
+// final too (forward: leading groups, adjoint: trailing groups).  One warp; its
+// lanes form the changes of groups lane and lane + 32.
+__device__ void advance_loop(LoopCtl& c) {
+    static_assert(kMaxG <= 64, "two groups per lane");
+    const int lane = threadIdx.x & 31;
+    double e[2];
+    unsigned below[2];
+    bool nan = false;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int g = lane + 32 * h;
+        double num = 0.0, den = 0.0;
+        if (g < c.G) {
+            num = __ldcg(c.res + 2 * g);
+            den = __ldcg(c.res + 2 * g + 1);
+        }
+        e[h] = den > 0.0 ? sqrt(num / den) : 0.0;
+        nan = nan || e[h] != e[h];
+        below[h] = __ballot_sync(0xffffffffu, e[h] < c.tol);
+    }
+    double eps = e[1] > e[0] ? e[1] : e[0];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const double o = __shfl_xor_sync(0xffffffffu, eps, off);
+        eps = o > eps ? o : eps;
+    }
+    if (__any_sync(0xffffffffu, nan)) eps = __longlong_as_double(0x7ff8000000000000LL);
+    if (lane != 0) return;
+    c.iters += 1;
+    c.resid = eps;
+    c.group_sweeps += c.use_window ? c.win[1] - c.win[0] : c.G;
+    c.swept[0] = c.win[0];
+    c.swept[1] = c.win[1];
+    if (eps < c.tol || c.iters >= c.max_iters) {
+        c.done = 1;
+    } else if (c.use_window) {
+        auto final_group = [&](int g) { return (below[g >> 5] >> (g & 31)) & 1u; };
+        if (!c.reverse)
+            while (c.win[0] < c.win[1] - 1 && final_group(c.win[0])) ++c.win[0];
+        else
+            while (c.win[1] - 1 > c.win[0] && final_group(c.win[1] - 1)) --c.win[1];
     }
 }
 
@@ -393,11 +454,17 @@ __global__ void __launch_bounds__(256) k_total_xs(size_t V, int G, const uint8_t
     }
 }
 
+// loop: the last block also advances the loop (a non-finite change ends it) and
+// leaves a copy of its state in pinned host memory.
 __global__ void __launch_bounds__(256) k_residual(size_t V, int M, const float* mom, float* prev,
-                                                  double* res, const int* skip, int g0, const int* win) {
+                                                  double* res, const int* skip, int g0, const int* win,
+                                                  LoopCtl* loop, LoopCtl* host_copy) {
     if (skip && *skip) return;
     const int g = g0 + blockIdx.y;
-    if (win && (g < win[0] || g >= win[1])) return;      // retired group (whole block)
+    if (win && (g < win[0] || g >= win[1])) {            // retired group (whole block)
+        if (!loop) return;
+        V = 0;
+    }
     double x[2] = {0.0, 0.0};
     // four voxels per thread and pass, their loads issued together
     const size_t stride = (size_t)gridDim.x * blockDim.x;
@@ -424,6 +491,23 @@ __global__ void __launch_bounds__(256) k_residual(size_t V, int M, const float* 
         x[1] += (double)cc;
     }
     block_reduce_add<2>(x, res + 2 * g);
+    if (loop && threadIdx.x < 32) {
+        __threadfence();                                 // this block's sums before its arrival
+        unsigned before = 0;
+        if (threadIdx.x == 0) before = atomicAdd(&loop->arrived, 1u);
+        before = __shfl_sync(0xffffffffu, before, 0);
+        if (before == gridDim.x * gridDim.y - 1) {
+            __threadfence();
+            advance_loop(*loop);
+            __syncwarp();
+            if (threadIdx.x == 0) {
+                if (!isfinite(loop->resid)) loop->done = 1;
+                loop->arrived = 0;
+                *host_copy = *loop;
+                __threadfence_system();
+            }
+        }
+    }
 }
 
 __global__ void __launch_bounds__(256) k_balance(size_t V, int G, int M, const uint8_t* mat,
@@ -472,45 +556,38 @@ __global__ void __launch_bounds__(256) k_zero(T* p, size_t n, const int* skip) {
         p[t] = T(0);
 }
 
-// One thread: update every live instance's iteration count and residual
-// (max over groups of sqrt(sum (dphi)^2 / sum phi^2)), retire it when the
-// relative change is below its tolerance or the cap is reached, and stop
-// the graph's while loop once all instances are retired.
-__global__ void k_decide(LoopCtl* ctl, int n, cudaGraphConditionalHandle h) {
-    if (threadIdx.x != 0) return;
+// One warp: advance every live instance and stop the graph's while loop once
+// all instances are retired.
+__global__ void __launch_bounds__(32) k_decide(LoopCtl* ctl, int n, cudaGraphConditionalHandle h) {
     bool all = true;
     for (int q = 0; q < n; ++q) {
-        LoopCtl& c = ctl[q];
-        if (c.done) continue;
-        double eps = 0.0;
-        for (int g = 0; g < c.G; ++g) {
-            const double num = c.res[2 * g], den = c.res[2 * g + 1];
-            const double e = den > 0.0 ? sqrt(num / den) : 0.0;
-            eps = e > eps || e != e ? e : eps;
-        }
-        c.iters += 1;
-        c.resid = eps;
-        c.group_sweeps += c.use_window ? c.win[1] - c.win[0] : c.G;
-        if (eps < c.tol || c.iters >= c.max_iters) {
-            c.done = 1;
-        } else {
-            all = false;
-            // shrink the active group window as the host loop does: a group whose
-            // relative change is below tol and whose sources are all final is
-            // final too (forward: leading groups, adjoint: trailing groups)
-            if (c.use_window) {
-                auto eps_of = [&](int g) {
-                    const double num = c.res[2 * g], den = c.res[2 * g + 1];
-                    return den > 0.0 ? sqrt(num / den) : 0.0;
-                };
-                if (!c.reverse)
-                    while (c.win[0] < c.win[1] - 1 && eps_of(c.win[0]) < c.tol) ++c.win[0];
-                else
-                    while (c.win[1] - 1 > c.win[0] && eps_of(c.win[1] - 1) < c.tol) --c.win[1];
-            }
-        }
+        const bool live = !ctl[q].done;
+        __syncwarp();
+        if (live) advance_loop(ctl[q]);
+        __syncwarp();
+        all = all && ctl[q].done;
     }
-    if (all) cudaGraphSetConditional(h, 0);
+    if (all && threadIdx.x == 0) cudaGraphSetConditional(h, 0);
+}
+
+// The window's moments and leakage and every residual sum to zero, in one
+// launch (per_group = V * M floats)
+__global__ void __launch_bounds__(256) k_zero_iteration(float* mom, size_t per_group, double* red, int G, const int* win,
+                                                        const int* skip) {
+    if (skip && *skip) return;
+    const int g0 = win[0], g1 = win[1];
+    const size_t first = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
+    const size_t beg = (size_t)g0 * per_group, end = (size_t)g1 * per_group;
+    // whole 16-byte vectors, then the unaligned ends
+    const size_t b4 = (beg + 3) / 4, e4 = end / 4;
+    float4* m4 = reinterpret_cast<float4*>(mom);
+    for (size_t t = b4 + first; t < e4; t += stride) m4[t] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (first < 4) {
+        if (beg + first < 4 * b4 && beg + first < end) mom[beg + first] = 0.0f;
+        if (4 * e4 + first < end && 4 * e4 >= beg) mom[4 * e4 + first] = 0.0f;
+    }
+    for (size_t g = first; g < (size_t)(2 * G); g += stride) red[G + g] = 0.0;
+    for (size_t g = g0 + first; g < (size_t)g1; g += stride) red[g] = 0.0;
 }
 
 template <class T>
@@ -530,9 +607,9 @@ unsigned blocks_for(size_t n, int bs, unsigned cap = 0) {
 }  // namespace
 
 // one resident wave of k_scatter_fast
-template <int GMAX, bool TR, bool HAS_BASE, bool ISO = false>
+template <int GMAX, bool TR, bool HAS_BASE, bool ISO = false, bool ZERO = false>
 cudaError_t launch_scatter_fast(const ScatterArgs& a, size_t smem, cudaStream_t s) {
-    auto kern = k_scatter_fast<GMAX, TR, HAS_BASE, ISO>;
+    auto kern = k_scatter_fast<GMAX, TR, HAS_BASE, ISO, ZERO>;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -556,6 +633,23 @@ cudaError_t launch_scatter_g(const ScatterArgs& a, cudaStream_t s) {
     const bool fast = fast_bytes <= kScatterTableSmem && a.phi && !a.iso_field && a.V * a.M < ((size_t)1 << 31);
     if (fast && a.iso && !a.transpose && !a.base)
         return launch_scatter_fast<GMAX, false, false, true>(a, fast_bytes, s);
+    if (a.zero_mom) {
+        // small moment arrays: zeroed by the threads that have read them, one launch
+        // fewer (16^3 cube, S4 P1: 0.86 -> 0.74 ms per solve together with the
+        // residual's last block deciding the loop); large ones in a launch of their
+        // own, which streams the stores (cylinder S8 P3, 160 MB: 16.5 ms against 17.2)
+        const bool small = a.V * a.M * a.G * sizeof(float) <= ((size_t)24 << 20);
+        if (small && fast && !a.iso && a.base)
+            return a.transpose ? launch_scatter_fast<GMAX, true, true, false, true>(a, fast_bytes, s)
+                               : launch_scatter_fast<GMAX, false, true, false, true>(a, fast_bytes, s);
+        ScatterArgs b = a;
+        b.zero_mom = nullptr;
+        cudaError_t e = launch_scatter_g<GMAX>(b, s);
+        if (e != cudaSuccess) return e;
+        k_zero_iteration<<<blocks_for((a.V * a.M * a.G + 15) / 16, 256, 152 * 8), 256, 0, s>>>(
+            a.zero_mom, a.V * a.M, a.zero_red, a.G, a.zero_win, a.skip);
+        return cudaGetLastError();
+    }
     if (fast && !a.iso) {
         if (a.transpose)
             return a.base ? launch_scatter_fast<GMAX, true, true>(a, fast_bytes, s)
@@ -590,10 +684,11 @@ cudaError_t launch_scatter(const ScatterArgs& a, cudaStream_t s) {
 }
 
 cudaError_t launch_residual(size_t V, int G, int M, const float* mom, float* prev, double* res,
-                            cudaStream_t s, const int* skip, int g0, int gcount, const int* win) {
+                            cudaStream_t s, const int* skip, int g0, int gcount, const int* win, LoopCtl* loop,
+                            LoopCtl* host_copy) {
     // sixteen voxels per thread (four passes)
     dim3 grid(blocks_for((V + 15) / 16, 256, 152), gcount < 0 ? G : gcount);
-    k_residual<<<grid, 256, 0, s>>>(V, M, mom, prev, res, skip, g0, win);
+    k_residual<<<grid, 256, 0, s>>>(V, M, mom, prev, res, skip, g0, win, loop, host_copy);
     return cudaGetLastError();
 }
 
