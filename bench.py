@@ -58,15 +58,12 @@ SWEEP_TRAFFIC = {
     (16, 16, 10, 1): (2246.4e6, "sweep_impl.cuh", "592eff4d10129e1bde8b55aecdf9fbf52f768e8c"),
     (16, 16, 5, 1): (1687.6e6, "sweep_impl.cuh", "592eff4d10129e1bde8b55aecdf9fbf52f768e8c"),
     (16, 8, 10, 3): (2534.9e6, "sweep_chain.cuh", "3502773d12d37fb58b50dbc1187553785b1df685"),
-    (8, 8, 10, 4): (3338.1e6, "sweep_flow.cuh", "19e106b753eb9e515798e72f9e5fe72303e29839"),
-    (16, 8, 10, 7): (2806.1e6, "sweep_flow.cuh", "19e106b753eb9e515798e72f9e5fe72303e29839"),
-    (8, 8, 10, 7): (3000.1e6, "sweep_flow.cuh", "19e106b753eb9e515798e72f9e5fe72303e29839"),
-    (16, 16, 10, 7): (2619.2e6, "sweep_flow.cuh", "19e106b753eb9e515798e72f9e5fe72303e29839"),
+    (8, 8, 10, 7): (2765.0e6, "sweep_flow.cuh", "82d92f9eaea4ab4b5e3147c1da7585970508598b"),
 }
 
 # sweep kernel by the library's sweep_kernel code
 SWEEP_KERNELS = {1: "k_sweep", 3: "k_sweep_chain", 4: "k_sweep_flow",
-                 5: "k_split_m2d + k_sweep_flow<split> + k_split_d2m", 7: "k_sweep_flow<face warp>",
+                 5: "k_split_m2d + k_sweep_flow<split> + k_split_d2m", 7: "k_sweep_flow",
                  8: "k_m2d_tc + k_sweep_flow<split> + k_d2m_tc"}
 
 # FP32 lanes per SM and SMs of a GB300 (the ALU roofline of the CUDA-core sweep)
