@@ -121,7 +121,7 @@ cudaError_t launch_uncollided_moments(const MomentArgs& a, cudaStream_t s);
 //                      + rho_v sum_g' sigma_s,l[mat v](g' -> g) phi[g'][v][lm]
 // (transpose: sigma_s,l(g -> g') instead, i.e. the adjoint's upscatter)
 // ---------------------------------------------------------------------------
-struct ScatterArgs {
+struct ScatterCore {
     size_t V;
     int G, M, L, nmat, transpose;
     const uint8_t* mat;
@@ -136,6 +136,10 @@ struct ScatterArgs {
     const int* skip;                   // if non-null and *skip != 0 the kernel does nothing
     int g0, g1;                        // destination groups updated: g0 .. g1 - 1 (g1 = 0: all)
     const int* win;                    // non-null: the window [win[0], win[1]) in device memory instead
+};
+// (the kernels that do not zero take the first part alone: with the whole block as their
+// parameter the 20-group forms spill)
+struct ScatterArgs : ScatterCore {
     float* zero_mom;                   // non-null (then phi itself): the groups of zero_win are zeroed once read,
     const int* zero_win;               // with their leakage zero_red[g] and every residual sum
     double* zero_red;                  // zero_red[G .. 3G)

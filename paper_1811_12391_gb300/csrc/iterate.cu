@@ -10,6 +10,7 @@
 // FP64, like the residual norm and the particle balance.
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "doctors_internal.h"
@@ -163,7 +164,7 @@ size_t scatter_table_bytes(const ScatterArgs& a) {
 }
 
 template <int GMAX>
-__global__ void __launch_bounds__(kScatterThreads, 3) k_scatter(const ScatterArgs a, int table_in_smem) {
+__global__ void __launch_bounds__(kScatterThreads, 3) k_scatter(const ScatterCore a, int table_in_smem) {
     extern __shared__ float tab_s[];
     if (a.skip && *a.skip) return;
     const int G = a.G;
@@ -275,7 +276,7 @@ size_t scatter_fast_table_bytes(const ScatterArgs& a) {
 }
 
 template <int GMAX, bool TR, bool HAS_BASE, bool ISO = false, bool ZERO = false>
-__global__ void __launch_bounds__(kScatterThreads, GMAX <= 24 ? 2 : 1) k_scatter_fast(const ScatterArgs a) {
+__global__ void __launch_bounds__(kScatterThreads, GMAX <= 24 ? 2 : 1) k_scatter_fast(const std::conditional_t<ZERO, ScatterArgs, ScatterCore> a) {
     extern __shared__ float4 tab4_s[];
     float* tab_s = reinterpret_cast<float*>(tab4_s);
     static_assert(GMAX % 4 == 0, "rows of whole 16-byte vectors");
@@ -291,10 +292,14 @@ __global__ void __launch_bounds__(kScatterThreads, GMAX <= 24 ? 2 : 1) k_scatter
     __syncthreads();
     const unsigned VM = (unsigned)(a.V * a.M), M = (unsigned)a.M;
     const int g_beg = a.win ? a.win[0] : a.g0, g_end = a.win ? a.win[1] : (a.g1 > 0 ? a.g1 : G);
-    const int z_beg = ZERO ? a.zero_win[0] : 0, z_end = ZERO ? a.zero_win[1] : 0;
-    if (ZERO && blockIdx.x == 0) {
-        for (int g = threadIdx.x; g < 2 * G; g += blockDim.x) a.zero_red[G + g] = 0.0;
-        for (int g = z_beg + threadIdx.x; g < z_end; g += blockDim.x) a.zero_red[g] = 0.0;
+    int z_beg = 0, z_end = 0;
+    if constexpr (ZERO) {
+        z_beg = a.zero_win[0];
+        z_end = a.zero_win[1];
+        if (blockIdx.x == 0) {
+            for (int g = threadIdx.x; g < 2 * G; g += blockDim.x) a.zero_red[G + g] = 0.0;
+            for (int g = z_beg + threadIdx.x; g < z_end; g += blockDim.x) a.zero_red[g] = 0.0;
+        }
     }
     const int L1 = a.L + 1;
     // no barrier below: threads leave the grid-stride loop independently
@@ -307,11 +312,12 @@ __global__ void __launch_bounds__(kScatterThreads, GMAX <= 24 ? 2 : 1) k_scatter
         const float* pp = a.phi + t;
 #pragma unroll
         for (int gp = 0; gp < GMAX; ++gp) {
-            const float* pg = pp + (size_t)(gp < G ? gp : G - 1) * VM;
-            const float x = ZERO ? *pg : __ldg(pg);
+            float x;
+            if constexpr (ZERO) x = pp[(size_t)(gp < G ? gp : G - 1) * VM];
+            else x = __ldg(pp + (size_t)(gp < G ? gp : G - 1) * VM);
             ph[gp] = gp < G ? x : 0.0f;
         }
-        if (ZERO) {
+        if constexpr (ZERO) {
             // read by no other thread: ready for the next sweep to add to
             float* pz = a.zero_mom + t;
 #pragma unroll
