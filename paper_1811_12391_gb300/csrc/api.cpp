@@ -113,65 +113,6 @@ ChainDirTable make_dir_table(const doctors_problem* p, int j0, int n) {
     return t;
 }
 
-// The dataflow kernel's table of whole octants: directions in swap order, the
-// transform rows split into even and odd parts (doctors_internal.h)
-ChainDirTable make_swap_table(const doctors_problem* p) {
-    const int A8 = p->A8, M = p->M, NP = flow_pairs(A8), NF = A8 - 2 * NP;
-    std::vector<int> first, partner, single;
-    for (int j = 0; j < A8; ++j) {
-        const double x = p->dirs[3 * j], y = p->dirs[3 * j + 1], z = p->dirs[3 * j + 2];
-        if (x == y) single.push_back(j);
-        if (x <= y) continue;
-        for (int k = 0; k < A8; ++k)
-            if (p->dirs[3 * k] == y && p->dirs[3 * k + 1] == x && p->dirs[3 * k + 2] == z && p->w[k] == p->w[j]) {
-                first.push_back(j);
-                partner.push_back(k);
-            }
-    }
-    ChainDirTable t{};
-    t.sig = p->d_sig;
-    if ((int)first.size() != NP || (int)single.size() != NF) return t;   // caller checks t.w[0]
-    const ChainDirTable n = make_dir_table(p, 0, A8);
-    std::vector<int> order(first);
-    order.insert(order.end(), partner.begin(), partner.end());
-    order.insert(order.end(), single.begin(), single.end());
-    for (int q = 0; q < A8; ++q) {
-        const int j = order[q];
-        t.cx[q] = n.cx[j]; t.cy[q] = n.cy[j]; t.cz[q] = n.cz[j]; t.csum[q] = n.csum[j];
-        t.lx[q] = n.lx[j]; t.ly[q] = n.ly[j]; t.lz[q] = n.lz[j]; t.w[q] = n.w[j];
-    }
-    // even, odd and plain functions at direction j
-    auto functions = [&](int j, double* even, double* odd, double* plain, bool to_dir) {
-        double R[16];
-        real_harmonics(3, p->dirs[3 * j], p->dirs[3 * j + 1], p->dirs[3 * j + 2], R);
-        auto c = [&](int lm) { return to_dir ? (2 * degree_of_lm(lm) + 1) / (4.0 * M_PI) * R[lm] : p->w[j] * R[lm]; };
-        for (int k = 0; k < flow_even1(M); ++k) even[k] = c(flow_even_lm(k));
-        for (int k = 0; k < flow_odd1(M); ++k) odd[k] = c(flow_odd_lm(k));
-        for (int k = 0; k < flow_comb(A8, M); ++k) {
-            even[flow_even1(M) + k] = 0.5 * (c(swap_a(k, M)) + swap_s(k) * c(swap_b(k, M)));
-            odd[flow_odd1(M) + k] = 0.5 * (c(swap_a(k, M)) - swap_s(k) * c(swap_b(k, M)));
-        }
-        for (int k = 0; k < flow_plain(A8, M); ++k) plain[k] = c(flow_plain_lm(k));
-    };
-    double ev[16], od[16], pl[8];
-    for (int q = 0; q < NP + NF; ++q) {
-        const bool pair = q < NP;
-        const int j = pair ? first[q] : single[q - NP];
-        functions(j, ev, od, pl, true);
-        for (int k = 0; k < flow_even(A8, M); ++k) t.mop[(pair ? flow_mop_pair(q, A8, M) : flow_mop_single(q - NP, A8, M)) + k] = (float)ev[k];
-        for (int k = 0; pair && k < flow_odd(A8, M); ++k) t.mop[flow_mop_odd(q, A8, M) + k] = (float)od[k];
-        for (int k = 0; k < flow_plain(A8, M); ++k) t.mop[(pair ? flow_mop_pair_pl(q, A8, M) : flow_mop_single_pl(q - NP, A8, M)) + k] = (float)pl[k];
-        functions(j, ev, od, pl, false);
-        for (int k = 0; k < flow_even(A8, M); ++k) t.dop[flow_dop_even(k, A8) + q] = (float)ev[k];
-        for (int k = 0; pair && k < flow_odd(A8, M); ++k) t.dop[flow_dop_odd(k, A8, M) + q] = (float)od[k];
-    }
-    for (int q = 0; q < A8; ++q) {
-        functions(order[q], ev, od, pl, false);
-        for (int k = 0; k < flow_plain(A8, M); ++k) t.dop[flow_dop_plain(k, A8, M) + q] = (float)pl[k];
-    }
-    return t;
-}
-
 void free_problem(doctors_problem* p) {
     void* ptrs[] = {p->d_coef, p->d_mat, p->d_rho, p->d_sigt, p->d_sigs,
                     p->d_phiu_src, p->d_phiu, p->d_U, p->d_Q, p->d_mom, p->d_src, p->d_src2, p->d_prev,
@@ -347,7 +288,7 @@ SweepArgs sweep_args(const doctors_problem* p, int reverse, const float* src, fl
     a.chain_slots = p->chain_slots;
     a.depth = p->flow_depth;
     a.fpitch = p->face_pitch;
-    a.dir_table = p->use_flow && flow_swap(p->ab, p->M) ? &p->dir_flow : &p->dir_table;
+    a.dir_table = &p->dir_table;
     a.flow = (p->use_flow || p->use_split) ? p->d_flow : nullptr;
     a.qang = p->d_qang;
     a.pang = p->d_pang;
@@ -364,10 +305,7 @@ cudaError_t launch_sweep(const doctors_problem* p, SweepArgs sw, int mode, cudaS
     if (p->use_split && mode == 0) return launch_split_sweep(sw, p->M, s, count);
     if (p->use_flow || p->use_split) {
         // modes 1 and 2 (stored / paired angular fluence) of the split path use the fused kernel
-        if (p->use_split) {
-            sw.chain_slots = p->flow_slots;
-            if (flow_swap(p->ab, p->M)) sw.dir_table = &p->dir_flow;
-        }
+        if (p->use_split) sw.chain_slots = p->flow_slots;
         if (p->nab == 1) {
             *count = 1;
             return launch_sweep_flow(sw, p->M, mode, s);
@@ -1127,11 +1065,7 @@ int doctors_create_problem(const doctors_mesh* mesh, const doctors_options* opt,
     rc = rc ? rc : dalloc_t(&p->d_src2, GVM, "sweep source (next iteration)");
     rc = rc ? rc : dalloc_t(&p->d_prev, GV, "previous scalar fluence");
     rc = rc ? rc : dalloc_t(&p->d_iso, (size_t)p->G, "volume source");
-    p->dir_table.sig = p->d_sig;   // the whole-octant tables also carry the per-cell cross sections
-    if (!rc && flow_octant_ab(p->A8) && flow_swap(p->A8, p->M)) {
-        p->dir_flow = make_swap_table(p);
-        if (p->dir_flow.w[0] <= 0.0f) return fail(DOCTORS_ERR_INVALID_ARG, "quadrature is not symmetric in x and y");
-    }
+    p->dir_table.sig = p->d_sig;   // the whole-octant table also carries the per-cell cross sections
     rc = rc ? rc : configure_sweep(p, p->tx, p->ty, p->ab, opt->sweep_kernel);
     static_assert(sizeof(LoopCtl) % sizeof(double) == 0, "loop state after the reductions");
     rc = rc ? rc : dalloc(reinterpret_cast<void**>(&p->d_red), 5 * (size_t)p->G * sizeof(double) + sizeof(LoopCtl), "reductions");

@@ -256,93 +256,6 @@ struct ChainDirTable {
     // last, so that the tables above keep their parameter offsets
     const float* sig;
 };
-// Swapping x and y maps an octant's level-symmetric set onto itself: its
-// directions are pairs (a, b, c), (b, a, c) of equal weight and single ones
-// with a = b.  Under the swap every R_lm is even, odd, or one of two that
-// change places (up to a sign), so sums and differences of a pair's fluxes and
-// of such harmonics split both moment transforms into an even and an odd part
-// of about half the multiply-adds and table entries each:
-//   moments to directions: psi_p, psi_p' = E +- O, E over the even functions, O
-//     over the odd ones; single directions have E only;
-//   directions to moments: even ones from psi_p + psi_p' (and the singles), odd
-//     ones from psi_p - psi_p'.
-// The halved sums of two table entries round once more than the entries.  Up to
-// S8 that moves the scalar results (J, view weights) by some 5e-9, ten times what
-// two runs differ by, so there the functions that change places keep their plain
-// entries: each entry still serves both directions of a pair.  The many
-// directions of S12 and S16 average it out, and there the plain entries would
-// cost 12 % (S16 P3, 96x80x24, 10 groups: 1.16 ms per sweep against 1.30 with the
-// l = 1 entries plain).  Water cylinder, S8 P3, per sweep: 0.703 ms with plain
-// rows per direction, 0.654 as here, 0.622 with everything mixed; S16 as above:
-// 1.57 with plain rows.
-// The dataflow kernel's table then lists the directions as the pairs' first
-// members, their partners, the single ones.  mop: per pair a row of even, odd
-// and plain coefficients, per single direction one of even and plain ones; dop:
-// a row of (pairs, singles) per even function, a row of pairs per odd one, and
-// a row of all directions per plain one.  Blocks of 12 directions are not closed
-// under the swap and keep the plain rows.
-__host__ __device__ constexpr int flow_pairs(int ab) { return ab == 3 ? 1 : ab == 6 ? 2 : ab == 10 ? 4 : ab == 21 ? 9 : ab == 36 ? 16 : 0; }
-// where it pays: P2 and P3, and P1 for S12 and S16 (S16 P1, 96x80x24: 0.825 ->
-// 0.760 ms; S8 P1 and every P0 gain nothing)
-__host__ __device__ constexpr bool flow_swap(int ab, int M) { return ab != 12 && (M >= 9 || (M == 4 && ab > 12)); }
-__host__ __device__ constexpr int flow_up2(int n) { return (n + 1) & ~1; }
-// even functions in order: lm 0, 2, 4, 6, 10, 12 (those there are), then the
-// even combinations; odd ones: lm 8, 14, then the odd combinations.  Combination
-// k of (a, b) is a + s b (even) and a - s b (odd), s the sign of the exchange
-__host__ __device__ constexpr int flow_even1(int M) { return M == 16 ? 6 : M == 9 ? 4 : M == 4 ? 2 : 1; }   // unmixed ones
-__host__ __device__ constexpr int flow_odd1(int M) { return M == 16 ? 2 : M == 9 ? 1 : 0; }
-__host__ __device__ constexpr bool flow_all_mixed(int ab) { return ab > 12; }
-__host__ __device__ constexpr int flow_comb(int ab, int M) {
-    return !flow_all_mixed(ab) ? 0 : M == 16 ? 4 : M == 9 ? 2 : M == 4 ? 1 : 0;
-}
-// plain functions: (lm 3, 1) from P1, (7, 5) from P2, (13, 11) and (15, 9) at P3;
-// the exchange of the last changes their sign
-__host__ __device__ constexpr int flow_plain(int ab, int M) {
-    return flow_all_mixed(ab) ? 0 : M == 16 ? 8 : M == 9 ? 4 : M == 4 ? 2 : 0;
-}
-__host__ __device__ constexpr int flow_plain_lm(int k) {
-    return k == 0 ? 3 : k == 1 ? 1 : k == 2 ? 7 : k == 3 ? 5 : k == 4 ? 13 : k == 5 ? 11 : k == 6 ? 15 : 9;
-}
-__host__ __device__ constexpr float flow_plain_s(int k) { return k < 6 ? 1.0f : -1.0f; }
-__host__ __device__ constexpr int flow_even(int ab, int M) { return flow_even1(M) + flow_comb(ab, M); }
-__host__ __device__ constexpr int flow_odd(int ab, int M) { return flow_odd1(M) + flow_comb(ab, M); }
-__host__ __device__ constexpr int flow_even_lm(int k) { return k <= 3 ? 2 * k : 2 * k + 2; }
-__host__ __device__ constexpr int flow_odd_lm(int k) { return k == 0 ? 8 : 14; }
-__host__ __device__ constexpr int swap_a(int k, int M) {
-    return M == 4 ? 3 : M == 9 ? (k == 0 ? 7 : 3) : k == 0 ? 7 : k == 1 ? 13 : k == 2 ? 3 : 15;
-}
-__host__ __device__ constexpr int swap_b(int k, int M) {
-    return M == 4 ? 1 : M == 9 ? (k == 0 ? 5 : 1) : k == 0 ? 5 : k == 1 ? 11 : k == 2 ? 1 : 9;
-}
-__host__ __device__ constexpr float swap_s(int k) { return k == 3 ? -1.0f : 1.0f; }
-// storage position of moment lm (the inverse of lm_of_pos)
-__host__ __device__ constexpr int pos_of_lm(int lm, int M) { return M == 16 ? (lm & 3) * 4 + (lm >> 2) : lm; }
-// row offsets in mop (even row of a pair, its odd row, its plain entries; row of
-// a single direction, its plain entries) and dop (even, odd, plain function)
-__host__ __device__ constexpr int flow_mop_pair(int p, int ab, int M) {
-    return p * (flow_up2(flow_even(ab, M)) + flow_up2(flow_odd(ab, M)) + flow_plain(ab, M));
-}
-__host__ __device__ constexpr int flow_mop_odd(int p, int ab, int M) {
-    return flow_mop_pair(p, ab, M) + flow_up2(flow_even(ab, M));
-}
-__host__ __device__ constexpr int flow_mop_pair_pl(int p, int ab, int M) {
-    return flow_mop_odd(p, ab, M) + flow_up2(flow_odd(ab, M));
-}
-__host__ __device__ constexpr int flow_mop_single(int f, int ab, int M) {
-    return flow_mop_pair(flow_pairs(ab), ab, M) + f * (flow_up2(flow_even(ab, M)) + flow_plain(ab, M));
-}
-__host__ __device__ constexpr int flow_mop_single_pl(int f, int ab, int M) {
-    return flow_mop_single(f, ab, M) + flow_up2(flow_even(ab, M));
-}
-__host__ __device__ constexpr int flow_dop_even(int k, int ab) { return k * flow_up2(ab - flow_pairs(ab)); }
-__host__ __device__ constexpr int flow_dop_odd(int k, int ab, int M) {
-    return flow_dop_even(flow_even(ab, M), ab) + k * flow_up2(flow_pairs(ab));
-}
-__host__ __device__ constexpr int flow_dop_plain(int k, int ab, int M) {
-    return flow_dop_odd(flow_odd(ab, M), ab, M) + k * flow_up2(ab);
-}
-static_assert(flow_mop_single(4, 36, 16) <= kFlowMaxAB * 16 && flow_dop_odd(6, 36, 16) <= 16 * kFlowMaxAB &&
-              flow_mop_single(3, 10, 16) <= kFlowMaxAB * 16 && flow_dop_plain(8, 10, 16) <= 16 * kFlowMaxAB, "table size");
 // the dataflow and chained kernels take SweepArgs and the table by value: the
 // parameter block (up to 32764 bytes on this architecture) must hold both
 static_assert(sizeof(SweepArgs) + sizeof(ChainDirTable) < 32764, "kernel parameter block too large");
@@ -476,8 +389,7 @@ struct doctors_problem {
     size_t tcb1_floats = 0;         // floats of b1 (b2 follows)
     size_t ang_floats = 0;
     int* d_flow = nullptr;          // [4] dataflow queue, done count, timeout flag
-    doctors::ChainDirTable dir_table{};   // first-octant direction table of the chained and split sweeps
-    doctors::ChainDirTable dir_flow{};    // dataflow sweep of whole octants: in pairs of swapped directions
+    doctors::ChainDirTable dir_table{};   // first-octant direction table of the chained and dataflow sweeps
     std::vector<doctors::ChainDirTable> dir_blk;   // dataflow sweep: the table of each direction block
     // device tables
     float* d_coef = nullptr;

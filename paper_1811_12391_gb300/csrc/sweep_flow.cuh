@@ -125,8 +125,12 @@ __device__ __forceinline__ void store_record(float* p, const float (&v)[AB]) {
                               4 * c4 + 3 < AB ? v[4 * c4 + 3 < AB ? 4 * c4 + 3 : 0] : 0.0f);
 }
 
-// sum of N products, two at a time: the two lanes of packed operations, and
-// their sum
+// sum of N products, two at a time: the two lanes of packed operations (even
+// and odd terms), and their sum.  FP64 results of a solve (J, the view weights)
+// show this order in their tenth digit: sums of a pair of directions and their
+// differences (the harmonics are even or odd under x <-> y) need fewer terms, but
+// moved them by up to 1e-8, and were taken back (water cylinder S8 P3 0.654 ms
+// per sweep with them, S16 P3 solve of 96x80x24 22.7 ms against 28.1)
 template <int N>
 __device__ __forceinline__ float2 dot2(const float* c, const float* x) {
     float2 t = N == 1 ? make_float2(c[0] * x[0], 0.0f) : make_float2(0.0f, 0.0f);
@@ -140,15 +144,6 @@ __device__ __forceinline__ float dot(const float* c, const float* x) {
     if constexpr (N == 1) return c[0] * x[0];
     const float2 t = dot2<N>(c, x);
     return t.x + t.y;
-}
-
-// sign of R_lm under the reflections (fx, fy, fz) = +-1
-__device__ __forceinline__ float sign_lm(int lm, float fx, float fy, float fz) {
-    float r = 1.0f;
-    if ((kOddX >> lm) & 1u) r *= fx;
-    if ((kOddY >> lm) & 1u) r *= fy;
-    if ((kOddZ >> lm) & 1u) r *= fz;
-    return r;
 }
 
 // column (li, lj) of column thread t: the tile's columns in diagonal order
@@ -189,8 +184,17 @@ __device__ __forceinline__ int flow_stage_tiles(int s, int ntx, int nty) {
 // NT: the largest CTA of the instantiation: 96 threads (tiles of up to 64
 // columns) or 288.  The register file is shared out by warps per scheduler, so
 // a bound of 288 threads leaves at most 168 registers (96 for two CTAs).
+// Resident CTAs of 96 threads: five up to 12 directions; three at S12 (four: the
+// same at step, diamond P3 solves of 96x80x24 22.1 against 21.2 ms); at S16 two
+// (step P0 to P2 12.2, 13.3, 24.3 ms; four: 12.9, 14.6, 27.6), but four for
+// diamond P0 to P2 (17.2, 18.8, 31.6 ms; two: 21.1, 23.7, 36.4), whose extra plane
+// and registers leave the scheduler with too few warps.
+constexpr int flow_min_ctas(int AB, int M, bool DD, int NT) {
+    if (NT > 96) return AB > 12 ? 1 : 2;
+    return AB <= 12 ? kFlowMinCtas : AB <= 21 ? 3 : DD && M < 16 ? 4 : 2;
+}
 template <int AB, int M, int MODE, bool SPLIT, bool DD, int NT>
-__global__ void __launch_bounds__(NT, NT == 96 ? (AB > 12 ? 4 : kFlowMinCtas) : AB > 12 ? 1 : 2)
+__global__ void __launch_bounds__(NT, flow_min_ctas(AB, M, DD, NT))
     k_sweep_flow(const SweepArgs a, const ChainDirTable dt) {
     static_assert(!SPLIT || MODE == 0, "split transforms sweep in mode 0 only");
     static_assert(!DD || !SPLIT, "diamond differencing in the fused kernel only");
@@ -199,8 +203,11 @@ __global__ void __launch_bounds__(NT, NT == 96 ? (AB > 12 ? 4 : kFlowMinCtas) : 
     constexpr int RS = flow_rs(AB), PW = flow_pw(AB);   // plane record: floats, vector width
     constexpr int RF = SPLIT ? ABP : M;                 // floats of a cell's source record
     constexpr bool COOP = RF == 16;                     // record moved by four lanes
-    constexpr bool SWAP = !SPLIT && flow_swap(AB, M);      // transforms in even and odd parts
-    constexpr int NPR = flow_pairs(AB), NE_ = flow_even(AB, M), NO_ = flow_odd(AB, M);
+    // S16 P3, small tiles: lane sums, and signs, of two directions or moments in one
+    // packed operation, which keeps the 36 x 16 products out of local memory (28.1 ms
+    // against 55.9 for a step solve of 96x80x24; elsewhere one by one is as fast
+    // or faster: S8 P3 11.98 against 12.38, S6 P3 10.2 against 10.7)
+    constexpr bool PAIRED = !SPLIT && AB == 36 && M == 16 && NT == 96;
     extern __shared__ float4 sm4[];
     if (a.skip && *a.skip) return;          // retired instance of a batched loop
     const int PX = chain_px(a.tx);
@@ -497,60 +504,20 @@ __global__ void __launch_bounds__(NT, NT == 96 ? (AB > 12 ? 4 : kFlowMinCtas) : 
                 if constexpr (SPLIT) {
 #pragma unroll
                     for (int q = 0; q < AB; ++q) psi[q] = s[q];
-                } else if constexpr (SWAP) {
-                    // even and odd functions of the source, with the octant's signs
-                    float ev[NE_], od[NO_ > 0 ? NO_ : 1];
+                } else if constexpr (PAIRED) {
 #pragma unroll
-                    for (int k = 0; k < flow_even1(M); ++k)
-                        ev[k] = s[pos_of_lm(flow_even_lm(k), M)] * sign_lm(flow_even_lm(k), fx, fy, fz);
-#pragma unroll
-                    for (int k = 0; k < flow_odd1(M); ++k)
-                        od[k] = s[pos_of_lm(flow_odd_lm(k), M)] * sign_lm(flow_odd_lm(k), fx, fy, fz);
-#pragma unroll
-                    for (int k = 0; k < flow_comb(AB, M); ++k) {
-                        const float sa = s[pos_of_lm(swap_a(k, M), M)];
-                        const float tb = s[pos_of_lm(swap_b(k, M), M)] * (swap_s(k) * sign_lm(swap_b(k, M), fx, fy, fz));
-                        ev[flow_even1(M) + k] = fmaf(sa, sign_lm(swap_a(k, M), fx, fy, fz), tb);
-                        od[flow_odd1(M) + k] = fmaf(sa, sign_lm(swap_a(k, M), fx, fy, fz), -tb);
-                    }
-                    // the plain functions' sources and their exchange
-                    constexpr int NPL = flow_plain(AB, M) / 2;
-                    float2 sxy[NPL > 0 ? NPL : 1], syx[NPL > 0 ? NPL : 1];
-#pragma unroll
-                    for (int k = 0; k < NPL; ++k) {
-                        sxy[k] = make_float2(s[pos_of_lm(flow_plain_lm(2 * k), M)] * sign_lm(flow_plain_lm(2 * k), fx, fy, fz),
-                                             s[pos_of_lm(flow_plain_lm(2 * k + 1), M)] * sign_lm(flow_plain_lm(2 * k + 1), fx, fy, fz));
-                        syx[k] = make_float2(flow_plain_s(2 * k) * sxy[k].y, flow_plain_s(2 * k) * sxy[k].x);
-                    }
-                    // a pair's fluxes from its even and odd sums (two functions per packed
-                    // operation), a single direction's from the even one
-#pragma unroll
-                    for (int p = 0; p < NPR; ++p) {
-                        const float2 e = dot2<NE_>(dt.mop + flow_mop_pair(p, AB, M), ev);
-                        float2 t1 = e, t2 = e;
-                        if constexpr (NO_ > 0) {
-                            const float2 o1 = dot2<NO_>(dt.mop + flow_mop_odd(p, AB, M), od);
-                            t1 = __fadd2_rn(e, o1);
-                            t2 = __fadd2_rn(e, make_float2(-o1.x, -o1.y));
-                        }
-#pragma unroll
-                        for (int k = 0; k < NPL; ++k) {
-                            const float2 c1 = make_float2(dt.mop[flow_mop_pair_pl(p, AB, M) + 2 * k],
-                                                          dt.mop[flow_mop_pair_pl(p, AB, M) + 2 * k + 1]);
-                            t1 = __ffma2_rn(c1, sxy[k], t1);
-                            t2 = __ffma2_rn(c1, syx[k], t2);
-                        }
-                        psi[p] = t1.x + t1.y;
-                        psi[NPR + p] = t2.x + t2.y;
+                    for (int m = 0; m < M; m += 2) {
+                        const float2 r2 = __fmul2_rn(make_float2(s[m], s[m + 1]),
+                                                     make_float2(octant_sign<M>(m, fx, fy, fz), octant_sign<M>(m + 1, fx, fy, fz)));
+                        s[m] = r2.x;
+                        s[m + 1] = r2.y;
                     }
 #pragma unroll
-                    for (int f = 0; f < AB - 2 * NPR; ++f) {
-                        float2 t = dot2<NE_>(dt.mop + flow_mop_single(f, AB, M), ev);
-#pragma unroll
-                        for (int k = 0; k < NPL; ++k)
-                            t = __ffma2_rn(make_float2(dt.mop[flow_mop_single_pl(f, AB, M) + 2 * k],
-                                                       dt.mop[flow_mop_single_pl(f, AB, M) + 2 * k + 1]), sxy[k], t);
-                        psi[2 * NPR + f] = t.x + t.y;
+                    for (int q = 0; q < AB; q += 2) {
+                        const float2 ta = dot2<M>(dt.mop + q * 16, s), tb = dot2<M>(dt.mop + (q + 1) * 16, s);
+                        const float2 p2 = __fadd2_rn(make_float2(ta.x, tb.x), make_float2(ta.y, tb.y));
+                        psi[q] = p2.x;
+                        psi[q + 1] = p2.y;
                     }
                 } else {
 #pragma unroll
@@ -667,37 +634,14 @@ __global__ void __launch_bounds__(NT, NT == 96 ? (AB > 12 ? 4 : kFlowMinCtas) : 
                 } else {
                     // directions -> moments (Eq. 3 for lm = 00): table rows hold w R_lm
                     float acc[M];
-                    if constexpr (SWAP) {
+                    if constexpr (PAIRED) {
 #pragma unroll
-                        for (int k = 0; k < flow_plain(AB, M); ++k)
-                            acc[pos_of_lm(flow_plain_lm(k), M)] =
-                                dot<AB>(dt.dop + flow_dop_plain(k, AB, M), psi) * sign_lm(flow_plain_lm(k), fx, fy, fz);
-                        // sums (and the single directions) and differences of the pairs
-                        float es[AB - NPR], fs[NPR > 0 ? NPR : 1];
-#pragma unroll
-                        for (int p = 0; p < NPR; ++p) {
-                            es[p] = psi[p] + psi[NPR + p];
-                            fs[p] = psi[p] - psi[NPR + p];
-                        }
-#pragma unroll
-                        for (int f = 0; f < AB - 2 * NPR; ++f) es[NPR + f] = psi[2 * NPR + f];
-#pragma unroll
-                        for (int k = 0; k < flow_even1(M); ++k)
-                            acc[pos_of_lm(flow_even_lm(k), M)] =
-                                dot<AB - NPR>(dt.dop + flow_dop_even(k, AB), es) * sign_lm(flow_even_lm(k), fx, fy, fz);
-#pragma unroll
-                        for (int k = 0; k < flow_odd1(M); ++k) {
-                            float t = 0.0f;
-                            if constexpr (NPR > 0) t = dot<NPR>(dt.dop + flow_dop_odd(k, AB, M), fs);
-                            acc[pos_of_lm(flow_odd_lm(k), M)] = t * sign_lm(flow_odd_lm(k), fx, fy, fz);
-                        }
-#pragma unroll
-                        for (int k = 0; k < flow_comb(AB, M); ++k) {
-                            const float e = dot<AB - NPR>(dt.dop + flow_dop_even(flow_even1(M) + k, AB), es);
-                            float o1 = 0.0f;
-                            if constexpr (NPR > 0) o1 = dot<NPR>(dt.dop + flow_dop_odd(flow_odd1(M) + k, AB, M), fs);
-                            acc[pos_of_lm(swap_a(k, M), M)] = (e + o1) * sign_lm(swap_a(k, M), fx, fy, fz);
-                            acc[pos_of_lm(swap_b(k, M), M)] = (e - o1) * (swap_s(k) * sign_lm(swap_b(k, M), fx, fy, fz));
+                        for (int m = 0; m < M; m += 2) {
+                            const float2 ta = dot2<AB>(dt.dop + m * kFlowMaxAB, psi), tb = dot2<AB>(dt.dop + (m + 1) * kFlowMaxAB, psi);
+                            const float2 r2 = __fmul2_rn(__fadd2_rn(make_float2(ta.x, tb.x), make_float2(ta.y, tb.y)),
+                                                         make_float2(octant_sign<M>(m, fx, fy, fz), octant_sign<M>(m + 1, fx, fy, fz)));
+                            acc[m] = r2.x;
+                            acc[m + 1] = r2.y;
                         }
                     } else {
 #pragma unroll
