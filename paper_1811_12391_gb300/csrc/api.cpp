@@ -1133,7 +1133,8 @@ int doctors_set_materials(doctors_problem* p, int n_mat, const uint8_t* mat, con
     CU(cudaMemcpyAsync(p->d_rho, hr.data(), p->V * sizeof(float), cudaMemcpyHostToDevice, p->stream));
     CU(cudaMemcpyAsync(p->d_sigt, st.data(), st.size() * sizeof(float), cudaMemcpyHostToDevice, p->stream));
     CU(cudaMemcpyAsync(p->d_sigs, ss.data(), ss.size() * sizeof(float), cudaMemcpyHostToDevice, p->stream));
-    CU(launch_total_xs(p->V, G, p->d_mat, p->d_rho, p->d_sigt, p->d_sig, p->stream));
+    CU(launch_total_xs(p->V, G, p->d_mat, flow_fused_sig(p->differencing == DOCTORS_DIFF_DIAMOND, p->M) ? nullptr : p->d_rho,
+                       p->d_sigt, p->d_sig, p->stream));
     CU(cudaStreamSynchronize(p->stream));
     p->nmat = n_mat;
     p->h_sigt.assign(sigma_t, sigma_t + (size_t)n_mat * G);

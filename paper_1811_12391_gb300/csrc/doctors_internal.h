@@ -152,7 +152,7 @@ cudaError_t launch_residual(size_t V, int G, int M, const float* mom, float* pre
                             const int* win = nullptr, struct LoopCtl* loop = nullptr, struct LoopCtl* host_copy = nullptr);
 // zero groups [win[0], win[1]) of a [G][per_group] float array unless *skip
 cudaError_t launch_zero_window(float* p, size_t per_group, int G, const int* win, const int* skip, cudaStream_t s);
-// out[g][v] = rho[v] * sigt[mat[v]][g] (FP32, the product the sweep forms)
+// out[g][v] = rho[v] * sigt[mat[v]][g] (FP32, the product the sweep forms; rho null: sigt alone)
 cudaError_t launch_total_xs(size_t V, int G, const uint8_t* mat, const float* rho, const float* sigt, float* out,
                             cudaStream_t s);
 cudaError_t launch_zero_window(double* p, size_t per_group, int G, const int* win, const int* skip, cudaStream_t s);
@@ -309,6 +309,12 @@ __host__ __device__ constexpr int flow_rs(int ab) {
     return flow_pw(ab) == 4 ? flow_abp_host(ab) : flow_pw(ab) == 2 ? (((ab + 1) / 2) | 1) * 2 : 1;
 }
 __host__ __device__ constexpr int flow_up4(int n) { return (n + 3) & ~3; }
+// Diamond sweeps of P0 and P2 form their denominators as fma(rho, sigma_t, sum c),
+// every other one as (rho sigma_t, rounded) + sum c.  Nothing but the results'
+// last digits depends on it: FP64 results (J, view weights) move by some 1e-9
+// where it changes.  The per-cell array then holds sigma_t at unit density and
+// the density is fetched beside it.
+__host__ __device__ constexpr bool flow_fused_sig(bool dd, int M) { return dd && M % 4 != 0; }
 // column threads in whole warps, then the face warp
 inline int flow_threads(int tx, int ty) { return ((tx * ty + 31) / 32 + 1) * 32; }
 // shared memory of one dataflow-sweep CTA: the source records (rf floats) and
@@ -318,7 +324,7 @@ inline int flow_threads(int tx, int ty) { return ((tx * ty + 31) / 32 + 1) * 32;
 // fluxes in separate planes), per-group leakage and the task slot
 inline size_t sweep_flow_smem_bytes(int ab, int rf, int tx, int ty, int gcount, int depth, bool dd = false) {
     const int T = tx * ty;
-    return 4 * ((size_t)flow_up4(depth * T * rf) + flow_up4(depth * T) + (size_t)depth * (tx + ty) * flow_abp_host(ab) +
+    return 4 * ((size_t)flow_up4(depth * T * rf) + flow_up4((flow_fused_sig(dd, rf) ? 2 : 1) * depth * T) + (size_t)depth * (tx + ty) * flow_abp_host(ab) +
                 flow_up4((dd ? 4 : 2) * chain_px(tx) * (ty + 1) * flow_rs(ab))) +
            8 * (size_t)gcount + 16;
 }
@@ -443,7 +449,7 @@ struct doctors_problem {
     double* h_acc = nullptr;       // pinned [2G]
     double* d_acc_src = nullptr;   // [S][G] per-source gradient sums (adjoint)
     double* h_acc_src = nullptr;   // pinned copy of it
-    float* d_sig = nullptr;        // [G][V] rho * sigma_t per cell and group (the dataflow sweep's one load)
+    float* d_sig = nullptr;        // [G][V] rho * sigma_t per cell and group (flow_fused_sig: sigma_t) for the dataflow sweep
     size_t acc_src_cap = 0;        // doubles in both
     // region-of-interest dose (allocated on first use)
     double* d_k = nullptr;         // [kMaxMat][G] dose factors

@@ -454,7 +454,7 @@ __device__ __forceinline__ void block_reduce_add(double (&x)[NV], double* dst) {
 __global__ void __launch_bounds__(256) k_total_xs(size_t V, int G, const uint8_t* mat, const float* rho,
                                                   const float* sigt, float* out) {
     for (size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (size_t)gridDim.x * blockDim.x) {
-        const float r = rho[v];
+        const float r = rho ? rho[v] : 1.0f;
         const int m = mat[v];
         for (int g = 0; g < G; ++g) out[(size_t)g * V + v] = r * __ldg(sigt + m * G + g);
     }

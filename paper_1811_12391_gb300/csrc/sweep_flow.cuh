@@ -208,6 +208,7 @@ __global__ void __launch_bounds__(NT, flow_min_ctas(AB, M, DD, NT))
     // against 55.9 for a step solve of 96x80x24; elsewhere one by one is as fast
     // or faster: S8 P3 11.98 against 12.38, S6 P3 10.2 against 10.7)
     constexpr bool PAIRED = !SPLIT && AB == 36 && M == 16 && NT == 96;
+    constexpr bool FUSED = !SPLIT && flow_fused_sig(DD, M);   // denominator fma(rho, sigma_t, sum c)
     extern __shared__ float4 sm4[];
     if (a.skip && *a.skip) return;          // retired instance of a batched loop
     const int PX = chain_px(a.tx);
@@ -215,8 +216,8 @@ __global__ void __launch_bounds__(NT, flow_min_ctas(AB, M, DD, NT))
     const int T = a.tx * a.ty;                                // column threads
     const int D = a.depth, PD = a.depth;    // steps held of source and face records (2 or 4)
     float* ring = reinterpret_cast<float*>(sm4);              // [D][T][RF] source records
-    float* sring = ring + flow_up4(D * T * RF);               // [D][T] rho sigma_t
-    float* landx = sring + flow_up4(D * T);                   // [PD][ty][ABP] fetched x-face records
+    float* sring = ring + flow_up4(D * T * RF);               // [D][T] rho sigma_t (FUSED: sigma_t, then [D][T] rho)
+    float* landx = sring + flow_up4((FUSED ? 2 : 1) * D * T);                   // [PD][ty][ABP] fetched x-face records
     float* landy = landx + PD * a.ty * ABP;                   // [PD][tx][ABP] fetched y-face records
     float* buf = landy + PD * a.tx * ABP;                     // [2][P][RS]
     float* bufy = DD ? buf + 2 * P * RS : buf;                // [2][P][RS] y-going faces (diamond)
@@ -463,6 +464,7 @@ __global__ void __launch_bounds__(NT, flow_min_ctas(AB, M, DD, NT))
                 }
             }
             if (pre) cp_async_f32(sring + slot * T + tid, sigg + vp);
+            if (FUSED && pre) cp_async_f32(sring + (D + slot) * T + tid, a.rho + vp);
             asm volatile("cp.async.commit_group;\n" ::: "memory");
         };
         for (int st = 0; st < D - 2; ++st) prefetch(st + 1, st & (D - 1));   // steps 0 .. D - 3
@@ -477,6 +479,7 @@ __global__ void __launch_bounds__(NT, flow_min_ctas(AB, M, DD, NT))
             if (act) {
                 const bool last = kr == a.nz - 1;
                 const float sig = sring[slot * T + tid];
+                const float rho = FUSED ? sring[(D + slot) * T + tid] : 1.0f;
                 const float* rs = ring + slot * T * RF;
                 float s[RF];
                 if constexpr (RF % 4 == 0) {
@@ -544,7 +547,9 @@ __global__ void __launch_bounds__(NT, flow_min_ctas(AB, M, DD, NT))
                                                    make_float2(psi[q], psi[q + 1]));
                             n2 = __ffma2_rn(make_float2(dt.cy[q], dt.cy[q + 1]), make_float2(py[e], py[e + 1]), n2);
                             n2 = __ffma2_rn(make_float2(dt.cz[q], dt.cz[q + 1]), make_float2(zc[q], zc[q + 1]), n2);
-                            const float2 d2 = __fadd2_rn(make_float2(sig, sig), make_float2(dt.csum[q], dt.csum[q + 1]));
+                            const float2 cs2 = make_float2(dt.csum[q], dt.csum[q + 1]);
+                            const float2 d2 = FUSED ? __ffma2_rn(make_float2(rho, rho), make_float2(sig, sig), cs2)
+                                                    : __fadd2_rn(make_float2(sig, sig), cs2);
                             psi[q] = n2.x * rcp_approx(d2.x);
                             psi[q + 1] = n2.y * rcp_approx(d2.y);
                         }
@@ -554,7 +559,7 @@ __global__ void __launch_bounds__(NT, flow_min_ctas(AB, M, DD, NT))
                             constexpr int q = AB - 1;
                             const int e = q - q0;
                             const float num = fmaf(dt.cz[q], zc[q], fmaf(dt.cy[q], py[e], fmaf(dt.cx[q], px[e], psi[q])));
-                            psi[q] = num * rcp_approx(sig + dt.csum[q]);
+                            psi[q] = num * rcp_approx(FUSED ? fmaf(rho, sig, dt.csum[q]) : sig + dt.csum[q]);
                         }
                     }
 #pragma unroll

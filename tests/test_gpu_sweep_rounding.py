@@ -85,3 +85,10 @@ def check(cases):
 @pytest.mark.parametrize("L", [0, 1, 2, 3])
 def test_bits(sn, L):
     check([c for c in CASES if c[:2] == (sn, L) and (c[2] == 0 or L in (1, 3))])
+
+
+@pytest.mark.parametrize("sn", [2, 4, 6, 8, 12, 16])
+@pytest.mark.parametrize("L", [0, 2])
+def test_bits_diamond_denominator(sn, L):
+    """P0 and P2 diamond cells: density times cross section is not rounded before the direction's term is added."""
+    check([c for c in CASES if c[:2] == (sn, L) and c[2] == 1])
