@@ -340,7 +340,8 @@ __global__ void __launch_bounds__(256) k_uncollided(const RayArgs base, const Ra
 #pragma unroll
                 for (int m = 0; m < kMaxMat; ++m)
                     if (m < r.nmat) tau = fmaf(s_sigt[m * r.G + g], lam[m], tau);
-                const float phi = __ldg(r.emit + (size_t)src[q].row * r.G + g) * expf(-tau) * inv;
+                // rounded before it is added, so that the total is the sum of the sources' fluences
+                const float phi = __fmul_rn(__ldg(r.emit + (size_t)src[q].row * r.G + g) * expf(-tau), inv);
                 tot[e] += phi;
 #pragma unroll
                 for (int m = 0; m < M; ++m) mom[e][m] = fmaf(phi, R[lm_of_pos(m, M)], mom[e][m]);
