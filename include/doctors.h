@@ -199,8 +199,9 @@ int doctors_set_source(doctors_problem *p, int n_src, const doctors_source *src)
  * collided problem (Eq. 2, vacuum boundaries) with step-differenced (or, per
  * options.differencing, diamond-differenced) octant wavefront sweeps, all
  * active groups per sweep.  Synchronises the stream.  Returns
- * DOCTORS_ERR_NOT_CONVERGED (results kept) if max_iters is reached.  `info`
- * may be NULL. */
+ * DOCTORS_ERR_NOT_CONVERGED (results kept) if max_iters is reached and
+ * DOCTORS_ERR_INVALID_ARG if a fluence is not finite (an emission weight *
+ * spectrum beyond FP32, for instance).  `info` may be NULL. */
 int doctors_solve(doctors_problem *p, doctors_result *info);
 
 /* Copy a group fluence [G][V] float32 (Eq. 3's scalar fluence; uncollided,

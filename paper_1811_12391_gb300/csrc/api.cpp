@@ -348,6 +348,19 @@ int check_flow(doctors_problem* p) {
     return DOCTORS_ERR_TIMEOUT;
 }
 
+// Ends a source iteration whose fluence is not finite.  A NaN flux looks like a
+// face record that is not written yet, so the sweep may have given up waits too:
+// the next solve of every problem starts from clean records.
+int non_finite(doctors_problem* const* ps, int n) {
+    for (int q = 0; q < n; ++q) {
+        CU(cudaStreamSynchronize(ps[q]->stream));
+        const int rc = check_flow(ps[q]);
+        if (rc && rc != DOCTORS_ERR_TIMEOUT) return rc;
+    }
+    set_error("source iteration produced a non-finite fluence");
+    return DOCTORS_ERR_INVALID_ARG;
+}
+
 // Source iteration: src = Q + S(mom); mom = sweep(src); residual.  `reverse`
 // selects the adjoint: sweep directions reversed and scattering transposed.
 int iterate(doctors_problem* p, int reverse, const float* Q, float* mom, doctors_result* info) {
@@ -438,11 +451,7 @@ int iterate(doctors_problem* p, int reverse, const float* Q, float* mom, doctors
         resid = c.resid;
         updates = (double)c.group_sweeps * (double)p->V * p->A;
         cur = (it - 1) & 1;
-        if (!std::isfinite(resid)) {
-            CU(cudaStreamSynchronize(p->stream));
-            set_error("source iteration produced a non-finite fluence");
-            return DOCTORS_ERR_INVALID_ARG;
-        }
+        if (!std::isfinite(resid)) return non_finite(&p, 1);
         conv = resid < tol;
     } else {
         // the other sweep kernels: the host reads the residuals and sets the window
@@ -484,12 +493,8 @@ int iterate(doctors_problem* p, int reverse, const float* Q, float* mom, doctors
             resid = 0.0;
             for (int g = g0; g < g1; ++g) {
                 const double num = p->h_red[p->G + 2 * g], den = p->h_red[p->G + 2 * g + 1];
-                eps[g] = den > 0.0 ? std::sqrt(num / den) : 0.0;
-                if (!std::isfinite(eps[g])) {
-                    CU(cudaStreamSynchronize(p->stream));
-                    set_error("source iteration produced a non-finite fluence");
-                    return DOCTORS_ERR_INVALID_ARG;
-                }
+                eps[g] = den == 0.0 ? 0.0 : std::sqrt(num / den);   // NaN sums stay NaN
+                if (!std::isfinite(eps[g])) return non_finite(&p, 1);
                 resid = std::max(resid, eps[g]);
             }
             if (resid < tol) {
@@ -671,10 +676,7 @@ int graph_iterate(doctors_problem** ps, int n, int reverse, const float* const* 
     for (int q = 0; q < n; ++q) max_it = std::max(max_it, ctl[q].iters);
     for (int q = 0; q < n; ++q) {
         doctors_problem* p = ps[q];
-        if (!std::isfinite(ctl[q].resid)) {
-            set_error("source iteration produced a non-finite fluence");
-            return DOCTORS_ERR_INVALID_ARG;
-        }
+        if (!std::isfinite(ctl[q].resid)) return non_finite(ps, n);
         // particle balance of the last sweep (FP64)
         const double vol = p->mesh.dx * p->mesh.dy * p->mesh.dz;
         double* d_bal = p->d_red + 3 * p->G;

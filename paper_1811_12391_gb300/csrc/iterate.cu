@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(kScatterThreads, GMAX <= 24 ? 2 : 1) k_scatter
 
 // Update a live instance's iteration count and residual (max over groups of
 // sqrt(sum (dphi)^2 / sum phi^2)), retire it when the relative change is below
-// its tolerance or the cap is reached, else shrink its active group window: a
+// its tolerance or not finite or the cap is reached, else shrink its active group window: a
 // group whose relative change is below tol and whose sources are all final is
 // final too (forward: leading groups, adjoint: trailing groups).  One warp; its
 // lanes form the changes of groups lane and lane + 32.
@@ -377,7 +377,7 @@ __device__ void advance_loop(LoopCtl& c) {
             num = __ldcg(c.res + 2 * g);
             den = __ldcg(c.res + 2 * g + 1);
         }
-        e[h] = den > 0.0 ? sqrt(num / den) : 0.0;
+        e[h] = den == 0.0 ? 0.0 : sqrt(num / den);       // NaN sums stay NaN
         nan = nan || e[h] != e[h];
         below[h] = __ballot_sync(0xffffffffu, e[h] < c.tol);
     }
@@ -394,7 +394,7 @@ __device__ void advance_loop(LoopCtl& c) {
     c.group_sweeps += c.use_window ? c.win[1] - c.win[0] : c.G;
     c.swept[0] = c.win[0];
     c.swept[1] = c.win[1];
-    if (eps < c.tol || c.iters >= c.max_iters) {
+    if (eps < c.tol || c.iters >= c.max_iters || !isfinite(eps)) {
         c.done = 1;
     } else if (c.use_window) {
         auto final_group = [&](int g) { return (below[g >> 5] >> (g & 31)) & 1u; };
@@ -460,8 +460,7 @@ __global__ void __launch_bounds__(256) k_total_xs(size_t V, int G, const uint8_t
     }
 }
 
-// loop: the last block also advances the loop (a non-finite change ends it) and
-// leaves a copy of its state in pinned host memory.
+// loop: the last block also advances the loop and leaves a copy of its state in pinned host memory.
 __global__ void __launch_bounds__(256) k_residual(size_t V, int M, const float* mom, float* prev,
                                                   double* res, const int* skip, int g0, const int* win,
                                                   LoopCtl* loop, LoopCtl* host_copy) {
@@ -507,7 +506,6 @@ __global__ void __launch_bounds__(256) k_residual(size_t V, int M, const float* 
             advance_loop(*loop);
             __syncwarp();
             if (threadIdx.x == 0) {
-                if (!isfinite(loop->resid)) loop->done = 1;
                 loop->arrived = 0;
                 *host_copy = *loop;
                 __threadfence_system();
