@@ -287,7 +287,6 @@ SweepArgs sweep_args(const doctors_problem* p, int reverse, const float* src, fl
     a.gcount = p->G;
     a.chain_slots = p->chain_slots;
     a.depth = p->flow_depth;
-    a.fpitch = p->face_pitch;
     a.dir_table = &p->dir_table;
     a.flow = (p->use_flow || p->use_split) ? p->d_flow : nullptr;
     a.qang = p->d_qang;
@@ -846,29 +845,24 @@ int configure_sweep(doctors_problem* p, int tx, int ty, int ab, int kernel) {
         return DOCTORS_ERR_INVALID_ARG;
     }
     // face buffers: [8][A/8][G][tiles-1][ny or nx][nz] per direction for the
-    // staged kernels; [8][G][tiles-1][ny or nx][nz] records of `pitch` floats for
-    // the dataflow kernels (unpadded records where padded ones do not fit)
-    int pitch = use_flow || use_split ? flow_face_pitch(ab) : flow_abp_host(p->A8);
-    for (;;) {
-        const size_t per_dir = std::max((size_t)p->A, (size_t)8 * std::max(pitch, flow_abp_host(p->A8)));
-        const size_t xf = per_dir * p->G * (ntx > 1 ? ntx - 1 : 0) * p->ny * p->nz;
-        const size_t yf = per_dir * p->G * (nty > 1 ? nty - 1 : 0) * p->nx * p->nz;
-        auto grow = [&](float** buf, size_t* bytes, size_t n, const char* what) -> int {
-            if (*buf != nullptr && n * sizeof(float) <= *bytes) return DOCTORS_OK;
-            float* nb = nullptr;
-            const int rc = dalloc_t(&nb, n, what);
-            if (rc) return rc;
-            if (*buf) cudaFree(*buf);
-            *buf = nb;
-            *bytes = n * sizeof(float);
-            return DOCTORS_OK;
-        };
-        int rc = grow(&p->d_xface, &p->xface_bytes, xf, "x face buffer");
-        if (!rc) rc = grow(&p->d_yface, &p->yface_bytes, yf, "y face buffer");
-        if (!rc) break;
-        if (rc != DOCTORS_ERR_OOM || pitch == flow_abp_host(ab)) return rc;
-        pitch = flow_abp_host(ab);
-    }
+    // staged kernels; [8][G][tiles-1][ny or nx][nz][A/8 padded to 4] records for
+    // the dataflow kernels
+    const size_t per_dir = std::max((size_t)p->A, (size_t)8 * flow_abp_host(p->A8));
+    const size_t xf = per_dir * p->G * (ntx > 1 ? ntx - 1 : 0) * p->ny * p->nz;
+    const size_t yf = per_dir * p->G * (nty > 1 ? nty - 1 : 0) * p->nx * p->nz;
+    auto grow = [&](float** buf, size_t* bytes, size_t n, const char* what) -> int {
+        if (*buf != nullptr && n * sizeof(float) <= *bytes) return DOCTORS_OK;
+        float* nb = nullptr;
+        const int rc = dalloc_t(&nb, n, what);
+        if (rc) return rc;
+        if (*buf) cudaFree(*buf);
+        *buf = nb;
+        *bytes = n * sizeof(float);
+        return DOCTORS_OK;
+    };
+    int rc = grow(&p->d_xface, &p->xface_bytes, xf, "x face buffer");
+    if (!rc) rc = grow(&p->d_yface, &p->yface_bytes, yf, "y face buffer");
+    if (rc) return rc;
     if (use_split) {
         // angular source and fluence records of every direction, group and voxel
         const size_t nang = (size_t)p->G * 8 * p->V * flow_abp_host(p->A8);
@@ -914,7 +908,6 @@ int configure_sweep(doctors_problem* p, int tx, int ty, int ab, int kernel) {
     p->chain_slots = chain_slots;
     p->flow_slots = flow_slots;
     p->flow_depth = flow_depth;
-    p->face_pitch = pitch;
     return DOCTORS_OK;
 }
 

@@ -215,7 +215,6 @@ struct SweepArgs {
     const int* skip;                   // if non-null and *skip != 0 the kernel does nothing
     int depth;                         // dataflow kernels: steps of source and face records held in shared memory
                                        // (fetched depth - 1 and depth steps ahead; 2 or 4)
-    int fpitch;                        // dataflow kernels: floats from one face record to the next
     int chain_slots;                   // > 0: chained kernel, at most this many CTAs per stage launch
     const int* win;                    // dataflow kernels: non-null: sweep the groups [win[0], win[1]) read from
                                        // device memory (g0, gcount then give only the buffer layout)
@@ -298,12 +297,6 @@ inline size_t sweep_chain_smem_bytes(int ab, int tx, int ty, int cmax, int gcoun
 // odd number of vectors, so the threads of a tile diagonal (an odd number of
 // records apart) fall in distinct shared-memory banks at that width.
 __host__ __device__ constexpr int flow_abp_host(int ab) { return (ab + 3) & ~3; }
-// floats from one face record to the next: whole 32-byte sectors for the
-// 16-byte records of S2 and S4 (a record that shares its sector with the one
-// its producer writes next is slow to read: S2 P0, 96x80x24, 10 groups takes
-// 0.331 ms per sweep at 16 bytes and 0.196 at 32; at 8 and more fluxes per
-// record padding only adds traffic: S8 P3 0.748 at 48 bytes, 0.760 at 64)
-__host__ __device__ constexpr int flow_face_pitch(int ab) { return ab <= 4 ? 8 : (ab + 3) & ~3; }
 __host__ __device__ constexpr int flow_pw(int ab) { return ab == 1 ? 1 : (flow_abp_host(ab) / 4) % 2 == 1 ? 4 : 2; }
 __host__ __device__ constexpr int flow_rs(int ab) {
     return flow_pw(ab) == 4 ? flow_abp_host(ab) : flow_pw(ab) == 2 ? (((ab + 1) / 2) | 1) * 2 : 1;
@@ -387,7 +380,6 @@ struct doctors_problem {
     bool flow_hw = false;           // dataflow sweep chosen as sweep_kernel 7 (the same kernel as 4)
     int differencing = 0;           // DOCTORS_DIFF_STEP or DOCTORS_DIFF_DIAMOND
     int flow_depth = 2;             // dataflow sweep: pipeline depth (SweepArgs::depth)
-    int face_pitch = 4;             // dataflow sweep: floats from one face record to the next
     int flow_slots = 0;             // CTA slots of the fused dataflow kernel (modes 1, 2 under split)
     float* d_qang = nullptr;        // [G][8][V][ABP] angular source (split)
     float* d_pang = nullptr;        // [G][8][V][ABP] angular fluence (split)

@@ -162,6 +162,18 @@ __device__ __forceinline__ void flow_column(int t, int tx, int ty, int& li, int&
     }
 }
 
+// place of plane k's face record in its column's run of nz.  The 16-byte records
+// of S2 and S4 lie two to a 32-byte sector, and one that shares its sector with
+// the one its producer writes next is slow to read: so the first and the second
+// half of the planes take the sectors' halves in turn, and a sector's two records
+// are nz / 2 steps apart
+template <int AB>
+__device__ __forceinline__ int flow_face_slot(int k, int nz) {
+    if constexpr (flow_abp(AB) > 4) return k;
+    const int half = (nz + 1) >> 1;
+    return k < half ? 2 * k : 2 * (k - half) + 1;
+}
+
 // tiles of stage s of an ntx x nty tile grid
 __device__ __forceinline__ int flow_stage_tiles(int s, int ntx, int nty) {
     const int lo = s - (nty - 1) > 0 ? s - (nty - 1) : 0;
@@ -199,7 +211,6 @@ __global__ void __launch_bounds__(NT, flow_min_ctas(AB, M, DD, NT))
     static_assert(!SPLIT || MODE == 0, "split transforms sweep in mode 0 only");
     static_assert(!DD || !SPLIT, "diamond differencing in the fused kernel only");
     constexpr int ABP = flow_abp(AB);
-    const int FP = AB <= 4 ? a.fpitch : ABP;            // floats between face records
     constexpr int RS = flow_rs(AB), PW = flow_pw(AB);   // plane record: floats, vector width
     constexpr int RF = SPLIT ? ABP : M;                 // floats of a cell's source record
     constexpr bool COOP = RF == 16;                     // record moved by four lanes
@@ -249,7 +260,7 @@ __global__ void __launch_bounds__(NT, flow_min_ctas(AB, M, DD, NT))
     const unsigned nxy = (unsigned)a.nx * a.ny;
     const size_t V = (size_t)nxy * a.nz;
     const int ntxf = a.ntx > 1 ? a.ntx - 1 : 0, ntyf = a.nty > 1 ? a.nty - 1 : 0;
-    const size_t xslab = (size_t)a.ny * a.nz * FP, yslab = (size_t)a.nx * a.nz * FP;
+    const size_t xslab = (size_t)a.ny * a.nz * ABP, yslab = (size_t)a.nx * a.nz * ABP;
     const int ntasks = a.ntx * a.nty * 8 * gcount;
     const int hend = a.nz + a.tx + a.ty - 2;                  // steps of a task
 
@@ -317,7 +328,7 @@ __global__ void __launch_bounds__(NT, flow_min_ctas(AB, M, DD, NT))
                     const int jr2 = bt * a.ty + q;
                     c.idx = q;
                     c.ok = jr2 < a.ny;
-                    c.src = at > 0 ? a.xface + (og * ntxf + at - 1) * xslab + (size_t)jr2 * a.nz * FP : nullptr;
+                    c.src = at > 0 ? a.xface + (og * ntxf + at - 1) * xslab + (size_t)jr2 * a.nz * ABP : nullptr;
                     c.land = (int)(landx - ring) + q * ABP;
                     c.lstride = a.ty * ABP;
                     c.halo = (int)(buf - ring) + (q + 1) * PX * RS;
@@ -325,7 +336,7 @@ __global__ void __launch_bounds__(NT, flow_min_ctas(AB, M, DD, NT))
                     c.idx = q - a.ty;
                     const int ir2 = at * a.tx + c.idx;
                     c.ok = ir2 < a.nx;
-                    c.src = bt > 0 ? a.yface + (og * ntyf + bt - 1) * yslab + (size_t)ir2 * a.nz * FP : nullptr;
+                    c.src = bt > 0 ? a.yface + (og * ntyf + bt - 1) * yslab + (size_t)ir2 * a.nz * ABP : nullptr;
                     c.land = (int)(landy - ring) + c.idx * ABP;
                     c.lstride = a.tx * ABP;
                     c.halo = (int)(bufy - ring) + (c.idx + 1) * RS;
@@ -340,7 +351,7 @@ __global__ void __launch_bounds__(NT, flow_min_ctas(AB, M, DD, NT))
                 const int pf = st - c.idx;
                 if (c.ok && c.src && (unsigned)pf < (unsigned)a.nz) {
                     float* land = ring + c.land + (st & (PD - 1)) * c.lstride;
-                    const float* s0 = c.src + (size_t)pf * FP;
+                    const float* s0 = c.src + (size_t)flow_face_slot<AB>(pf, a.nz) * ABP;
 #pragma unroll
                     for (int c4 = 0; c4 < ABP / 4; ++c4) cp_async_cg16(land + 4 * c4, s0 + 4 * c4);
                 }
@@ -363,7 +374,7 @@ __global__ void __launch_bounds__(NT, flow_min_ctas(AB, M, DD, NT))
                     for (int q = 0; q < ABP; ++q) v[q] = 0.0f;
                 } else {
                     const float4* land = reinterpret_cast<const float4*>(ring + c.land + (st & (PD - 1)) * c.lstride);
-                    float* s0 = c.src + (size_t)pf * FP;
+                    float* s0 = c.src + (size_t)flow_face_slot<AB>(pf, a.nz) * ABP;
 #pragma unroll
                     for (int c4 = 0; c4 < ABP / 4; ++c4) {
                         const float4 t4 = land[c4];
@@ -425,8 +436,8 @@ __global__ void __launch_bounds__(NT, flow_min_ctas(AB, M, DD, NT))
         const bool xout = li == a.tx - 1 && at < a.ntx - 1 && !withhold;
         const bool yout = lj == a.ty - 1 && bt < a.nty - 1 && !withhold;
         const bool xleak = ir == a.nx - 1, yleak = jr == a.ny - 1;
-        float* const xo = a.xface + (og * ntxf + at) * xslab + (size_t)jr * a.nz * FP;
-        float* const yo = a.yface + (og * ntyf + bt) * yslab + (size_t)ir * a.nz * FP;
+        float* const xo = a.xface + (og * ntxf + at) * xslab + (size_t)jr * a.nz * ABP;
+        float* const yo = a.yface + (og * ntyf + bt) * yslab + (size_t)ir * a.nz * ABP;
         const size_t ang0 = ((size_t)g * 8 + oe) * V;       // angular records of (group, direction octant)
         const float* const srcg = SPLIT ? a.qang + ang0 * ABP : a.src + gV * M;
         const float* const sigg = dt.sig + gV;
@@ -604,12 +615,12 @@ __global__ void __launch_bounds__(NT, flow_min_ctas(AB, M, DD, NT))
                     if (xout) {
 #pragma unroll
                         for (int q = 0; q < AB; ++q) f[q] = fxo[q];
-                        store_record<AB>(xo + (size_t)kr * FP, f);
+                        store_record<AB>(xo + (size_t)flow_face_slot<AB>(kr, a.nz) * ABP, f);
                     }
                     if (yout) {
 #pragma unroll
                         for (int q = 0; q < AB; ++q) f[q] = fyo[q];
-                        store_record<AB>(yo + (size_t)kr * FP, f);
+                        store_record<AB>(yo + (size_t)flow_face_slot<AB>(kr, a.nz) * ABP, f);
                     }
                     if (xleak || yleak || last) {
 #pragma unroll
@@ -620,8 +631,8 @@ __global__ void __launch_bounds__(NT, flow_min_ctas(AB, M, DD, NT))
                         }
                     }
                 } else {
-                    if (xout) store_record<AB>(xo + (size_t)kr * FP, psi);
-                    if (yout) store_record<AB>(yo + (size_t)kr * FP, psi);
+                    if (xout) store_record<AB>(xo + (size_t)flow_face_slot<AB>(kr, a.nz) * ABP, psi);
+                    if (yout) store_record<AB>(yo + (size_t)flow_face_slot<AB>(kr, a.nz) * ABP, psi);
                     if (xleak || yleak || last) {
 #pragma unroll
                         for (int q = 0; q < AB; ++q) {
@@ -831,7 +842,7 @@ template <int M>
 cudaError_t launch_split_sweep_m(const SweepArgs& a, cudaStream_t s, int* count) {
     *count = 0;
     if (a.gcount <= 0) return cudaSuccess;
-    if (a.dir_table == nullptr || a.flow == nullptr || a.dir_table->sig == nullptr || (a.depth != 2 && a.depth != 4) || a.fpitch < flow_abp(a.ab) || a.nab != 1 || !a.qang ||
+    if (a.dir_table == nullptr || a.flow == nullptr || a.dir_table->sig == nullptr || (a.depth != 2 && a.depth != 4) || a.nab != 1 || !a.qang ||
         !a.pang)
         return cudaErrorInvalidValue;
     const size_t V = (size_t)a.nx * a.ny * a.nz;
@@ -887,7 +898,7 @@ cudaError_t launch_split_sweep_m(const SweepArgs& a, cudaStream_t s, int* count)
 template <int M, int MODE>
 cudaError_t launch_sweep_flow_m(const SweepArgs& a, cudaStream_t s) {
     if (a.gcount <= 0) return cudaSuccess;
-    if (a.dir_table == nullptr || a.flow == nullptr || a.dir_table->sig == nullptr || (a.depth != 2 && a.depth != 4) || a.fpitch < flow_abp(a.ab) || a.blk < 0 || a.blk >= a.nab ||
+    if (a.dir_table == nullptr || a.flow == nullptr || a.dir_table->sig == nullptr || (a.depth != 2 && a.depth != 4) || a.blk < 0 || a.blk >= a.nab ||
         a.ab * a.nab != a.A8)
         return cudaErrorInvalidValue;
     const bool dd = a.dd != 0;
