@@ -165,7 +165,8 @@ typedef struct doctors_result {
     double ms_iterate;       /* device time of the source iteration */
     double ms_sweep;         /* device time of the sweep launches alone (summed over iterations) */
     double ms_total;         /* device time of the whole call */
-    long long launches;      /* kernels launched by the call */
+    long long launches;      /* kernels launched by the call (those enqueued past the last iteration, which
+                                return at once, included) */
 } doctors_result;
 
 typedef struct doctors_problem doctors_problem;

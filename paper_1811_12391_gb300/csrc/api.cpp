@@ -425,8 +425,9 @@ int iterate(doctors_problem* p, int reverse, const float* Q, float* mom, doctors
             CU(cudaEventRecord(ev[2], p->stream));
             if (i + 1 < p->opt.max_iters) {
                 sa.out = srcs[(i + 1) & 1];
-                CU(launch_scatter(sa, p->stream));
-                ++p->launches;
+                int ns = 0;
+                CU(launch_scatter(sa, p->stream, &ns));
+                p->launches += ns;
             }
             p->launches += nl + 1;
             return DOCTORS_OK;
@@ -588,7 +589,7 @@ int graph_iterate(doctors_problem** ps, int n, int reverse, const float* const* 
         e = cudaGraphAddNode(&node, graph, nullptr, nullptr, 0, &cp);
         if (e == cudaSuccess) body = cp.conditional.phGraph_out[0];
     }
-    long long per_iter_launches = 1;
+    std::vector<long long> per_iter(n, 0);   // kernels of an instance in the loop's body
     // independent instances run on parallel branches of the body: the
     // capture forks onto up to kBranches side streams and joins before the
     // decision kernel
@@ -640,7 +641,8 @@ int graph_iterate(doctors_problem** ps, int n, int reverse, const float* const* 
             if (e == cudaSuccess) e = launch_sweep(p, sw, 0, cs, &nl);
             if (e == cudaSuccess)
                 e = launch_residual(p->V, p->G, p->M, moms[q], p->d_prev, p->d_red + p->G, cs, skip, 0, -1, win);
-            per_iter_launches += 4 + nl;
+            // scattering, zeroing (moments, leakage, sums), sweep, residual
+            per_iter[q] = (p->use_split ? 4 : 5) + nl;
         }
         if (nb > 1) {
             for (int b = 0; b < nb && e == cudaSuccess; ++b) {
@@ -699,7 +701,7 @@ int graph_iterate(doctors_problem** ps, int n, int reverse, const float* const* 
             r.cell_updates = (double)ctl[q].group_sweeps * (double)p->V * p->A;
             r.ms_sweep = -1.0;   // not separable inside the graph
         }
-        p->launches += (long long)max_it * per_iter_launches / n + 1;
+        p->launches += max_it * (per_iter[q] + (q == 0 ? 1 : 0)) + 1;   // the decision kernel counts with the first
         if (!conv) worst = DOCTORS_ERR_NOT_CONVERGED;
     }
     return worst;

@@ -144,7 +144,8 @@ struct ScatterArgs : ScatterCore {
     const int* zero_win;               // with their leakage zero_red[g] and every residual sum
     double* zero_red;                  // zero_red[G .. 3G)
 };
-cudaError_t launch_scatter(const ScatterArgs& a, cudaStream_t s);
+// *count: kernels launched (two where the zeroing has a launch of its own)
+cudaError_t launch_scatter(const ScatterArgs& a, cudaStream_t s, int* count = nullptr);
 
 // residual: res[g][0] += sum_v (phi00 - prev)^2, res[g][1] += sum_v phi00^2; prev = phi00
 cudaError_t launch_residual(size_t V, int G, int M, const float* mom, float* prev, double* res,

@@ -629,7 +629,7 @@ cudaError_t launch_scatter_fast(const ScatterArgs& a, size_t smem, cudaStream_t 
 }
 
 template <int GMAX>
-cudaError_t launch_scatter_g(const ScatterArgs& a, cudaStream_t s) {
+cudaError_t launch_scatter_g(const ScatterArgs& a, cudaStream_t s, int* count) {
     const size_t tab_bytes = scatter_table_bytes<GMAX>(a);
     const int staged = tab_bytes <= kScatterTableSmem ? 1 : 0;
     const size_t smem = staged ? tab_bytes : 0;
@@ -648,8 +648,9 @@ cudaError_t launch_scatter_g(const ScatterArgs& a, cudaStream_t s) {
                                : launch_scatter_fast<GMAX, false, true, false, true>(a, fast_bytes, s);
         ScatterArgs b = a;
         b.zero_mom = nullptr;
-        cudaError_t e = launch_scatter_g<GMAX>(b, s);
+        cudaError_t e = launch_scatter_g<GMAX>(b, s, nullptr);
         if (e != cudaSuccess) return e;
+        if (count) *count = 2;
         k_zero_iteration<<<blocks_for((a.V * a.M * a.G + 15) / 16, 256, 152 * 8), 256, 0, s>>>(
             a.zero_mom, a.V * a.M, a.zero_red, a.G, a.zero_win, a.skip);
         return cudaGetLastError();
@@ -669,7 +670,8 @@ cudaError_t launch_scatter_g(const ScatterArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_scatter(const ScatterArgs& a, cudaStream_t s) {
+cudaError_t launch_scatter(const ScatterArgs& a, cudaStream_t s, int* count) {
+    if (count) *count = 1;
     if (!a.phi && !a.base && !a.iso && a.iso_field && !a.skip && !a.win && a.g0 == 0 && (a.g1 == 0 || a.g1 == a.G)) {
         const size_t GV = (size_t)a.G * a.V;
         if (a.M % 4 == 0)
@@ -678,12 +680,12 @@ cudaError_t launch_scatter(const ScatterArgs& a, cudaStream_t s) {
             k_iso_source<1><<<blocks_for(GV * a.M, 256, 152 * 16), 256, 0, s>>>(GV, a.M, a.iso_field, a.iso_field_scale, a.out);
         return cudaGetLastError();
     }
-    if (a.G <= 8) return launch_scatter_g<8>(a, s);
-    if (a.G <= 16) return launch_scatter_g<16>(a, s);
-    if (a.G <= 20) return launch_scatter_g<20>(a, s);
-    if (a.G <= 24) return launch_scatter_g<24>(a, s);
-    if (a.G <= 32) return launch_scatter_g<32>(a, s);
-    if (a.G <= 64) return launch_scatter_g<64>(a, s);
+    if (a.G <= 8) return launch_scatter_g<8>(a, s, count);
+    if (a.G <= 16) return launch_scatter_g<16>(a, s, count);
+    if (a.G <= 20) return launch_scatter_g<20>(a, s, count);
+    if (a.G <= 24) return launch_scatter_g<24>(a, s, count);
+    if (a.G <= 32) return launch_scatter_g<32>(a, s, count);
+    if (a.G <= 64) return launch_scatter_g<64>(a, s, count);
     return cudaErrorInvalidValue;
 }
 
