@@ -287,6 +287,7 @@ SweepArgs sweep_args(const doctors_problem* p, int reverse, const float* src, fl
     a.gcount = p->G;
     a.chain_slots = p->chain_slots;
     a.depth = p->flow_depth;
+    a.fdepth = p->face_depth;
     a.dir_table = &p->dir_table;
     a.flow = (p->use_flow || p->use_split) ? p->d_flow : nullptr;
     a.qang = p->d_qang;
@@ -776,7 +777,7 @@ int configure_sweep(doctors_problem* p, int tx, int ty, int ab, int kernel) {
         return DOCTORS_ERR_INVALID_ARG;
     }
     const int ntx = (p->nx + tx - 1) / tx, nty = (p->ny + ty - 1) / ty;
-    int chain_slots = 0, flow_slots = 0, flow_depth = 2;
+    int chain_slots = 0, flow_slots = 0, flow_depth = 2, face_depth = 2;
     size_t smem = 0;
     if (use_flow || use_split) {
         int sms = 0;
@@ -789,12 +790,17 @@ int configure_sweep(doctors_problem* p, int tx, int ty, int ab, int kernel) {
         const int threads = flow_threads(tx, ty);
         int per_sm = 0, per_sm_main = 0;
         const int rf_split = flow_abp_host(ab);
-        auto fused = [&](int depth) { return sweep_flow_smem_bytes(ab, p->M, tx, ty, p->G, depth, dd); };
-        auto split = [&](int depth) { return use_split ? sweep_flow_smem_bytes(ab, rf_split, tx, ty, p->G, depth) : (size_t)0; };
+        auto fused = [&](int depth) { return sweep_flow_smem_bytes(ab, p->M, tx, ty, p->G, depth, depth == 2 ? face_depth : depth, dd); };
+        auto split = [&](int depth) {
+            return use_split ? sweep_flow_smem_bytes(ab, rf_split, tx, ty, p->G, depth, depth == 2 ? face_depth : depth) : (size_t)0;
+        };
         auto query = [&](int depth, int* b, int* bm) {
             *b = sweep_flow_blocks_per_sm(ab, p->M, threads, fused(depth), false, dd);
             *bm = use_split ? sweep_flow_blocks_per_sm(ab, p->M, threads, split(depth), true) : *b;
         };
+        // where two steps of face records do not fit beside two of source records
+        // (diamond S12 P3 in tiles of one column by 224 and more), one step's do
+        if (std::max(fused(2), split(2)) > 227 * 1024) face_depth = 1;
         smem = std::max(fused(2), split(2));
         if (std::max(fused(4), split(4)) <= 227 * 1024) {
             query(4, &per_sm, &per_sm_main);
@@ -812,6 +818,7 @@ int configure_sweep(doctors_problem* p, int tx, int ty, int ab, int kernel) {
                 flow_depth = 2;
             }
         }
+        if (flow_depth == 4) face_depth = 4;
         if (smem <= 227 * 1024) {
             if (per_sm < 1 || per_sm_main < 1) {
                 set_error("dataflow sweep cannot be resident with this tile");
@@ -910,6 +917,7 @@ int configure_sweep(doctors_problem* p, int tx, int ty, int ab, int kernel) {
     p->chain_slots = chain_slots;
     p->flow_slots = flow_slots;
     p->flow_depth = flow_depth;
+    p->face_depth = face_depth;
     return DOCTORS_OK;
 }
 

@@ -214,8 +214,9 @@ struct SweepArgs {
     float* psi;                        // written (mode 1) or read (mode 2): [G][V][A], dataflow kernel [G][8][V][nab][ABP]
     float* prod;                       // [G][V]: mode 2 accumulator
     const int* skip;                   // if non-null and *skip != 0 the kernel does nothing
-    int depth;                         // dataflow kernels: steps of source and face records held in shared memory
-                                       // (fetched depth - 1 and depth steps ahead; 2 or 4)
+    int depth;                         // dataflow kernels: steps of source records held in shared memory (2 or 4;
+                                       // fetched depth - 1 steps ahead)
+    int fdepth;                        // ... and of face records (the same, or 1; fetched that many steps ahead)
     int chain_slots;                   // > 0: chained kernel, at most this many CTAs per stage launch
     const int* win;                    // dataflow kernels: non-null: sweep the groups [win[0], win[1]) read from
                                        // device memory (g0, gcount then give only the buffer layout)
@@ -311,14 +312,14 @@ __host__ __device__ constexpr int flow_up4(int n) { return (n + 3) & ~3; }
 __host__ __device__ constexpr bool flow_fused_sig(bool dd, int M) { return dd && M % 4 != 0; }
 // column threads in whole warps, then the face warp
 inline int flow_threads(int tx, int ty) { return ((tx * ty + 31) / 32 + 1) * 32; }
+inline bool flow_depths_ok(int depth, int fdepth) { return (depth == 2 || depth == 4) && (fdepth == depth || fdepth == 1); }
 // shared memory of one dataflow-sweep CTA: the source records (rf floats) and
 // cross sections of `depth` steps, the fetched face records of the tile's
-// first row and column of as many steps, two
-// halo-padded hyperplanes (diamond differencing: x-going and y-going face
+// first row and column of `fdepth` steps, two halo-padded hyperplanes (diamond differencing: x-going and y-going face
 // fluxes in separate planes), per-group leakage and the task slot
-inline size_t sweep_flow_smem_bytes(int ab, int rf, int tx, int ty, int gcount, int depth, bool dd = false) {
+inline size_t sweep_flow_smem_bytes(int ab, int rf, int tx, int ty, int gcount, int depth, int fdepth, bool dd = false) {
     const int T = tx * ty;
-    return 4 * ((size_t)flow_up4(depth * T * rf) + flow_up4((flow_fused_sig(dd, rf) ? 2 : 1) * depth * T) + (size_t)depth * (tx + ty) * flow_abp_host(ab) +
+    return 4 * ((size_t)flow_up4(depth * T * rf) + flow_up4((flow_fused_sig(dd, rf) ? 2 : 1) * depth * T) + (size_t)fdepth * (tx + ty) * flow_abp_host(ab) +
                 flow_up4((dd ? 4 : 2) * chain_px(tx) * (ty + 1) * flow_rs(ab))) +
            8 * (size_t)gcount + 16;
 }
@@ -380,7 +381,8 @@ struct doctors_problem {
     bool split_tc = false;          // ... those passes on the tensor cores (P3)
     bool flow_hw = false;           // dataflow sweep chosen as sweep_kernel 7 (the same kernel as 4)
     int differencing = 0;           // DOCTORS_DIFF_STEP or DOCTORS_DIFF_DIAMOND
-    int flow_depth = 2;             // dataflow sweep: pipeline depth (SweepArgs::depth)
+    int flow_depth = 2;             // dataflow sweep: pipeline depths (SweepArgs::depth, fdepth)
+    int face_depth = 2;
     int flow_slots = 0;             // CTA slots of the fused dataflow kernel (modes 1, 2 under split)
     float* d_qang = nullptr;        // [G][8][V][ABP] angular source (split)
     float* d_pang = nullptr;        // [G][8][V][ABP] angular fluence (split)

@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(NT, flow_min_ctas(AB, M, DD, NT))
     const int PX = chain_px(a.tx);
     const int P = PX * (a.ty + 1);
     const int T = a.tx * a.ty;                                // column threads
-    const int D = a.depth, PD = a.depth;    // steps held of source and face records (2 or 4)
+    const int D = a.depth, PD = a.fdepth;   // steps held of source records (2 or 4) and of face records (also 1)
     float* ring = reinterpret_cast<float*>(sm4);              // [D][T][RF] source records
     float* sring = ring + flow_up4(D * T * RF);               // [D][T] rho sigma_t (FUSED: sigma_t, then [D][T] rho)
     float* landx = sring + flow_up4((FUSED ? 2 : 1) * D * T);                   // [PD][ty][ABP] fetched x-face records
@@ -412,7 +412,8 @@ __global__ void __launch_bounds__(NT, flow_min_ctas(AB, M, DD, NT))
                 if (h == htake && lane == 0) next = atomicAdd(a.flow + 0, 1);
                 issue(h + PD);
                 if (PD == 4) asm volatile("cp.async.wait_group 3;\n" ::: "memory");
-                else asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+                else if (PD == 2) asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+                else asm volatile("cp.async.wait_group 0;\n" ::: "memory");
                 fill1(first, h + 1, h & 1);
                 for (int q = lane + 32; q < nrec; q += 32) fill1(rec(q), h + 1, h & 1);
                 if (h == hgive && lane == 0) *task_s = next;
@@ -842,7 +843,7 @@ template <int M>
 cudaError_t launch_split_sweep_m(const SweepArgs& a, cudaStream_t s, int* count) {
     *count = 0;
     if (a.gcount <= 0) return cudaSuccess;
-    if (a.dir_table == nullptr || a.flow == nullptr || a.dir_table->sig == nullptr || (a.depth != 2 && a.depth != 4) || a.nab != 1 || !a.qang ||
+    if (a.dir_table == nullptr || a.flow == nullptr || a.dir_table->sig == nullptr || !flow_depths_ok(a.depth, a.fdepth) || a.nab != 1 || !a.qang ||
         !a.pang)
         return cudaErrorInvalidValue;
     const size_t V = (size_t)a.nx * a.ny * a.nz;
@@ -858,7 +859,7 @@ cudaError_t launch_split_sweep_m(const SweepArgs& a, cudaStream_t s, int* count)
     const int slots = std::max(1, a.chain_slots / std::max(1, a.slot_share));
     const int grid = ntasks < slots ? ntasks : slots;
     const int T = flow_threads(a.tx, a.ty);
-    const size_t smem = sweep_flow_smem_bytes(a.ab, flow_abp(a.ab), a.tx, a.ty, a.gcount, a.depth);
+    const size_t smem = sweep_flow_smem_bytes(a.ab, flow_abp(a.ab), a.tx, a.ty, a.gcount, a.depth, a.fdepth);
     cudaError_t e = cudaSuccess;
     // P3: the transforms on the tensor cores when the problem holds their tables
     const bool tc = M == 16 && a.tc_b1 && a.tc_b2;
@@ -898,7 +899,7 @@ cudaError_t launch_split_sweep_m(const SweepArgs& a, cudaStream_t s, int* count)
 template <int M, int MODE>
 cudaError_t launch_sweep_flow_m(const SweepArgs& a, cudaStream_t s) {
     if (a.gcount <= 0) return cudaSuccess;
-    if (a.dir_table == nullptr || a.flow == nullptr || a.dir_table->sig == nullptr || (a.depth != 2 && a.depth != 4) || a.blk < 0 || a.blk >= a.nab ||
+    if (a.dir_table == nullptr || a.flow == nullptr || a.dir_table->sig == nullptr || !flow_depths_ok(a.depth, a.fdepth) || a.blk < 0 || a.blk >= a.nab ||
         a.ab * a.nab != a.A8)
         return cudaErrorInvalidValue;
     const bool dd = a.dd != 0;
@@ -912,7 +913,7 @@ cudaError_t launch_sweep_flow_m(const SweepArgs& a, cudaStream_t s) {
     const int slots = std::max(1, a.chain_slots / std::max(1, a.slot_share));
     const int grid = ntasks < slots ? ntasks : slots;
     const int T = flow_threads(a.tx, a.ty);
-    const size_t smem = sweep_flow_smem_bytes(a.ab, M, a.tx, a.ty, a.gcount, a.depth, dd);
+    const size_t smem = sweep_flow_smem_bytes(a.ab, M, a.tx, a.ty, a.gcount, a.depth, a.fdepth, dd);
     cudaError_t e = cudaSuccess;
     auto launch = [&](auto kern) {
         if (smem > 48 * 1024) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
