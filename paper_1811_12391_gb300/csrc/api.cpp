@@ -1361,9 +1361,10 @@ int doctors_solve_batch(doctors_problem** problems, int n, doctors_result* resul
         problems[q]->solved = false;
         problems[q]->adjoint_done = false;
         problems[q]->launches = 0;
-        CU(cudaStreamSynchronize(p0->stream));
         rc = first_collision(problems[q]);
         if (rc) return rc;
+        // the problem's own stream, which the loop on the first one's does not follow
+        CU(cudaStreamSynchronize(problems[q]->stream));
     }
     CU(cudaEventRecord(p0->ev[1], p0->stream));
     std::vector<const float*> Qs(n);
