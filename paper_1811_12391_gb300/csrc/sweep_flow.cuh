@@ -194,13 +194,17 @@ __device__ __forceinline__ int flow_stage_tiles(int s, int ntx, int nty) {
 // records and the leakage carry the face fluxes, not the cell flux.
 //
 // NT: the largest CTA of the instantiation: 96 threads (tiles of up to 64
-// columns) or 288.  The register file is shared out by warps per scheduler, so
+// columns) or 288 (one has 160, flow_mid_cta).  The register file is shared out by warps per scheduler, so
 // a bound of 288 threads leaves at most 168 registers (96 for two CTAs).
 // Resident CTAs of 96 threads: five up to 12 directions; three at S12 (four: the
 // same at step, diamond P3 solves of 96x80x24 22.1 against 21.2 ms); at S16 two
 // (step P0 to P2 12.2, 13.3, 24.3 ms; four: 12.9, 14.6, 27.6), but four for
 // diamond P0 to P2 (17.2, 18.8, 31.6 ms; two: 21.1, 23.7, 36.4), whose extra plane
 // and registers leave the scheduler with too few warps.
+// Step S16 P3 has a third instantiation, for 97 to 160 threads (tiles of up to 128
+// columns): two warps per scheduler leave it 255 registers (16x8 tiles, six
+// iterations of 64x60x20, 8 groups: 5.0 ms, 7.2 with the bound for 288 threads).
+constexpr bool flow_mid_cta(int AB, int M, int threads, bool DD) { return AB == 36 && M == 16 && !DD && threads > 96 && threads <= 160; }
 constexpr int flow_min_ctas(int AB, int M, bool DD, int NT) {
     if (NT > 96) return AB > 12 ? 1 : 2;
     return AB <= 12 ? kFlowMinCtas : AB <= 21 ? 3 : DD && M < 16 ? 4 : 2;
@@ -214,11 +218,13 @@ __global__ void __launch_bounds__(NT, flow_min_ctas(AB, M, DD, NT))
     constexpr int RS = flow_rs(AB), PW = flow_pw(AB);   // plane record: floats, vector width
     constexpr int RF = SPLIT ? ABP : M;                 // floats of a cell's source record
     constexpr bool COOP = RF == 16;                     // record moved by four lanes
-    // S16 P3, small tiles: lane sums, and signs, of two directions or moments in one
-    // packed operation, which keeps the 36 x 16 products out of local memory (28.1 ms
-    // against 55.9 for a step solve of 96x80x24; elsewhere one by one is as fast
-    // or faster: S8 P3 11.98 against 12.38, S6 P3 10.2 against 10.7)
-    constexpr bool PAIRED = !SPLIT && AB == 36 && M == 16 && NT == 96;
+    // S16 P3: lane sums, and signs, of two directions or moments in one packed
+    // operation, which keeps the 36 x 16 products out of local memory (28.1 ms
+    // against 55.9 for a step solve of 96x80x24; six iterations of 64x60x20 diamond,
+    // 16x16 tiles: 8.1 against 11.4).  Not in step CTAs of up to 288 threads, whose
+    // 168 registers it overflows (16x16 tiles 9.8 against 7.3); elsewhere one by one
+    // is as fast or faster (S8 P3 11.98 against 12.38, S6 P3 10.2 against 10.7)
+    constexpr bool PAIRED = !SPLIT && AB == 36 && M == 16 && (DD || NT < 288);
     constexpr bool FUSED = !SPLIT && flow_fused_sig(DD, M);   // denominator fma(rho, sigma_t, sum c)
     extern __shared__ float4 sm4[];
     if (a.skip && *a.skip) return;          // retired instance of a batched loop
@@ -821,6 +827,8 @@ int sweep_flow_blocks_per_sm(int ab, int threads, size_t smem, bool split, bool 
         } else if (threads <= 96) {                                                 \
             if (dd) query(k_sweep_flow<AB, M, 0, false, true, 96>);                  \
             else query(k_sweep_flow<AB, M, 0, false, false, 96>);                    \
+        } else if (flow_mid_cta(AB, M, threads, dd)) {                               \
+            if constexpr (flow_mid_cta(AB, M, 160, false)) query(k_sweep_flow<AB, M, 0, false, false, 160>); \
         } else if (dd) query(k_sweep_flow<AB, M, 0, false, true, 288>);              \
         else query(k_sweep_flow<AB, M, 0, false, false, 288>);                       \
         break;
@@ -924,6 +932,8 @@ cudaError_t launch_sweep_flow_m(const SweepArgs& a, cudaStream_t s) {
         if (T <= 96) {                                                               \
             if (dd) launch(k_sweep_flow<AB, M, MODE, false, true, 96>);               \
             else launch(k_sweep_flow<AB, M, MODE, false, false, 96>);                 \
+        } else if (flow_mid_cta(AB, M, T, dd)) {                                     \
+            if constexpr (flow_mid_cta(AB, M, 160, false)) launch(k_sweep_flow<AB, M, MODE, false, false, 160>); \
         } else if (dd) launch(k_sweep_flow<AB, M, MODE, false, true, 288>);           \
         else launch(k_sweep_flow<AB, M, MODE, false, false, 288>);                    \
         break;

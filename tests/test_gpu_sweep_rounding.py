@@ -75,7 +75,7 @@ def check(cases):
     for c in cases:
         want = golden[key(*c)], golden[key(*c) + "_gradients"]
         assert np.count_nonzero(want[0]) > 0.9 * want[0].size
-        for tile in ((0, 0), (3, 2), (10, 8)):
+        for tile in ((0, 0), (3, 2), (10, 8), (16, 10)):
             for w, got in zip(want, results(*c, tile=tile)):
                 np.testing.assert_array_equal(got.view(f"u{got.itemsize}"), w.view(f"u{w.itemsize}"),
                                               err_msg=str((key(*c), tile)))
