@@ -632,12 +632,18 @@ int graph_iterate(doctors_problem** ps, int n, int reverse, const float* const* 
             SweepArgs sw = sweep_args(p, reverse, p->d_src, moms[q]);
             sw.skip = skip;
             sw.win = win;
-            // two instances' dataflow sweeps share the resident CTA slots, so
-            // one's wavefront fill and drain overlap the other's full stages
-            // (measured on the axial-scan batch: sharing among 2, 4 and 8 took
-            // 2025, 2058 and 2233 ms against 2038 ms without sharing; more
-            // instances at once spill each other's working sets out of L2)
-            sw.slot_share = std::min(nb, 2);
+            // two instances' dataflow sweeps share the resident CTA slots where one
+            // fills them at most four times over, so that one's wavefront fill and
+            // drain overlap the other's full stages (batches of 4 to 8, 8 groups, ms
+            // shared / not: 48x48x24 S6 P1 7.90 / 8.67, S8 P2 19.9 / 20.8; 64x64x32 S4
+            // P3 17.6 / 17.1, 96x96x48 S6 P1 27.3 / 22.9).  Not with large direction
+            // tables, which two launches on one SM read from the constant cache in turn
+            // (S8 P3, 19 groups, 24x24x12 12.5 / 11.7, 64x64x32 67.4 / 57.7; S12 P1
+            // 48x48x24 16.6 / 15.3, S16 P1 27.4 / 20.1).  More than two spill each
+            // other's working sets out of L2
+            const long long tasks = 8LL * p->ntx * p->nty * p->G;
+            const bool share = p->ab <= 12 && p->ab * p->M <= 96 && tasks <= 4LL * p->chain_slots;
+            sw.slot_share = share ? std::min(nb, 2) : 1;
             int nl = 0;
             if (e == cudaSuccess) e = launch_sweep(p, sw, 0, cs, &nl);
             if (e == cudaSuccess)
@@ -977,9 +983,11 @@ int doctors_create_problem(const doctors_mesh* mesh, const doctors_options* opt,
     // tile costs more than the longer fill of a 16 x 16 tile, unless its ragged
     // edge sweeps many more columns (8 x 8 -> 16 x 16, ms per sweep: 64x64x16 S6 P0
     // 0.106 -> 0.094, S8 P1 0.153 -> 0.140, 256x256x64 S6 P0 3.03 -> 2.79, 75x61x37
-    // S4 P1 0.260 -> 0.236, 20x150x12 S6 P0 0.122 -> 0.108; but 40x33x20, where it
-    // sweeps 1.44 times the columns, S6 P1 0.077 -> 0.083; with P3 64x64x32 S8 0.63
-    // -> 0.78, with S12 and S16 1.2 to 1.4 times slower)
+    // S4 P1 0.260 -> 0.236, 20x150x12 S6 P0 0.122 -> 0.108, 96x80x24 S2 P0 0.205 ->
+    // 0.171, diamond 0.225 -> 0.206, 128x128x64 S4 P1 diamond 1.05 -> 0.96, though P0
+    // 1.10 -> 1.16; but 40x33x20, where it sweeps 1.44 times the columns, S6 P1 0.077
+    // -> 0.083; with P3 64x64x32 S8 0.67 -> 0.86, with S12 and S16 1.2 to 1.6 times
+    // slower)
     int tdef = flow_default ? 8 : 16;
     if (flow_default && p->A8 == p->ab && p->M <= 4 && p->ab <= 10 && opt->tile_x <= 0 && opt->tile_y <= 0) {
         auto columns = [&](int t) {
