@@ -339,7 +339,7 @@ int doctors_quadrature(int sn_order, int legendre, double *dirs, double *w, doub
  * concurrent projections).  After each problem's ray trace, one CUDA graph
  * holds every problem's source iteration inside a device-side while loop:
  * per iteration, every live problem's scattering source, all its wavefront
- * stages and its FP64 residual, then a one-thread decision that retires the
+ * stages and its FP64 residual, then a decision that retires the
  * problems that have converged (their kernels return at entry from then on)
  * and ends the loop when all are retired.  Everything runs on the first
  * problem's stream; all problems must be on one device and have materials

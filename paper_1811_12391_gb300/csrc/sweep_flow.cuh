@@ -50,6 +50,10 @@
 //     CTAs of 288 threads (96 registers) the cooperative addresses spilled in
 //     the 8x8 tile too (0.748 against 0.703 ms; six CTAs of 96 registers spill
 //     and take 0.930, four of up to 168 take 0.742).
+// Together, average over a solve: cylinder 0.97 -> 0.68 ms per sweep, diamond 0.77;
+// the abdomen (128x128x48, S16 P3, 19 groups) 12.0 -> 10.0.  A P3 step is bound by
+// the issue of its instructions (about a quarter of them packed FMAs), a P0 or P1
+// step on a small mesh by the latency of its chain.
 #pragma once
 
 #include <algorithm>
@@ -129,8 +133,8 @@ __device__ __forceinline__ void store_record(float* p, const float (&v)[AB]) {
 // and odd terms), and their sum.  FP64 results of a solve (J, the view weights)
 // show this order in their tenth digit: sums of a pair of directions and their
 // differences (the harmonics are even or odd under x <-> y) need fewer terms, but
-// moved them by up to 1e-8, and were taken back (water cylinder S8 P3 0.654 ms
-// per sweep with them, S16 P3 solve of 96x80x24 22.7 ms against 28.1)
+// moved them by up to 1e-8 and were taken back (with them a sweep of the cylinder
+// took 4 % less, a S16 P3 solve of 96x80x24 22.7 ms instead of 28.1)
 template <int N>
 __device__ __forceinline__ float2 dot2(const float* c, const float* x) {
     float2 t = N == 1 ? make_float2(c[0] * x[0], 0.0f) : make_float2(0.0f, 0.0f);
