@@ -58,7 +58,7 @@ SWEEP_TRAFFIC = {
     (16, 16, 10, 1): (2246.4e6, "sweep_impl.cuh", "592eff4d10129e1bde8b55aecdf9fbf52f768e8c"),
     (16, 16, 5, 1): (1687.6e6, "sweep_impl.cuh", "592eff4d10129e1bde8b55aecdf9fbf52f768e8c"),
     (16, 8, 10, 3): (2534.9e6, "sweep_chain.cuh", "3502773d12d37fb58b50dbc1187553785b1df685"),
-    (8, 8, 10, 7): (2765.0e6, "sweep_flow.cuh", "82d92f9eaea4ab4b5e3147c1da7585970508598b"),
+    (8, 8, 10, 7): (2772.0e6, "sweep_flow.cuh", "ddedd7513448b3fac9d728b4eecac131fd316500"),
 }
 
 # sweep kernel by the library's sweep_kernel code

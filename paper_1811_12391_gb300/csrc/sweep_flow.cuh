@@ -200,11 +200,12 @@ __device__ __forceinline__ int flow_stage_tiles(int s, int ntx, int nty) {
 // NT: the largest CTA of the instantiation: 96 threads (tiles of up to 64
 // columns) or 288 (one has 160, flow_mid_cta).  The register file is shared out by warps per scheduler, so
 // a bound of 288 threads leaves at most 168 registers (96 for two CTAs).
-// Resident CTAs of 96 threads: five up to 12 directions; three at S12 (four: the
-// same at step, diamond P3 solves of 96x80x24 22.1 against 21.2 ms); at S16 two
-// (step P0 to P2 12.2, 13.3, 24.3 ms; four: 12.9, 14.6, 27.6), but four for
-// diamond P0 to P2 (17.2, 18.8, 31.6 ms; two: 21.1, 23.7, 36.4), whose extra plane
-// and registers leave the scheduler with too few warps.
+// The bound of the instantiations for 96 threads, in CTAs per SM: five up to 12
+// directions; three at S12 (four: the same at step, diamond P3 solves of 96x80x24
+// 22.1 against 21.2 ms); at S16 two (step P0 to P2 12.2, 13.3, 24.3 ms; four: 12.9,
+// 14.6, 27.6; step P3 takes 166 registers, so four CTAs are resident all the same),
+// but four for diamond P0 to P2 (17.2, 18.8, 31.6 ms; two: 21.1, 23.7, 36.4), which
+// otherwise take so many registers that too few warps are resident.
 // Step S16 P3 has a third instantiation, for 97 to 160 threads (tiles of up to 128
 // columns): two warps per scheduler leave it 255 registers (16x8 tiles, six
 // iterations of 64x60x20, 8 groups: 5.0 ms, 7.2 with the bound for 288 threads).
