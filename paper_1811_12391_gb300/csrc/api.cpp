@@ -1605,6 +1605,7 @@ int adjoint_impl(doctors_problem* p, const double* response, int mem, const RoiT
     if (rc) return rc;
     const size_t GV = (size_t)p->G * p->V, GVM = GV * p->M;
     p->launches = 0;
+    p->adjoint_done = false;
     CU(cudaEventRecord(p->ev[0], p->stream));
     if (roi) {
         CU(launch_roi_response(p->V, p->G, p->d_mat, p->d_rho, roi->k, roi->roi, p->d_r, p->d_rf, p->stream));

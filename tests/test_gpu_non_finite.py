@@ -71,6 +71,9 @@ def test_batch_and_adjoint(tile):
     with pytest.raises(C.DoctorsError) as e:
         hs[0].roi_gradients(p.k_dep, roi * 1e45)
     assert e.value.code == C.DOCTORS_ERR_INVALID_ARG
+    with pytest.raises(C.DoctorsError) as e:     # the adjoint fluence of the call before is overwritten
+        hs[0].fluence_host(C.DOCTORS_FLUENCE_ADJOINT)
+    assert e.value.code == C.DOCTORS_ERR_STATE
     again = hs[0].roi_gradients(p.k_dep, roi)
     np.testing.assert_allclose(again["weights"].cpu().numpy(), g["weights"].cpu().numpy(), rtol=REL_TOL)
     for h in hs:
